@@ -86,6 +86,29 @@ struct __align__(16) SpreadWarpSmem {  // 16-byte aligned: staged rows take vect
     short perm[kFastCap];  // canonical position -> slot in the tile
 };
 
+// Canonical order (by original index) of the c <= kFastCap sites from slot s0:
+// perm[r] = the slot of rank r.  The rank of a site is the number of sites
+// with a smaller index (keys compared four at a time, from 16-byte broadcast
+// loads); keys is padded to a multiple of 4 with values above every index.
+__device__ __forceinline__ void rank_tile(int* keys, short* perm, const int* __restrict__ sorig, int s0, int c) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < c; i += 32) keys[i] = __ldg(&sorig[s0 + i]);
+    if (lane < ((c + 3) & ~3) - c) keys[c + lane] = INT_MAX;
+    __syncwarp();
+    const int c4 = (c + 3) >> 2;
+    const int4* k4 = reinterpret_cast<const int4*>(keys);
+    for (int i = lane; i < c; i += 32) {
+        const int ki = keys[i];
+        int r = 0;
+        for (int j = 0; j < c4; ++j) {
+            const int4 kk = k4[j];
+            r += (kk.x < ki) + (kk.y < ki) + (kk.z < ki) + (kk.w < ki);
+        }
+        perm[r] = (short)i;
+    }
+    __syncwarp();
+}
+
 // One tile by one warp: rank its sites, spread them in canonical order into
 // the warp's shared patch, write the patch out.  Ends with __syncwarp, after
 // which the warp may start on its next tile.
@@ -103,11 +126,6 @@ __device__ __forceinline__ void spread_tile(int tile, SpreadWarpSmem<T, P, TILE>
     const int s0 = tr.x;
     const int c = tr.y - s0;
     const bool ranked = c > 1 && c <= kFastCap;
-    if (ranked) {
-        for (int i = lane; i < c; i += 32) W.u.keys[i] = __ldg(&sorig[s0 + i]);
-        // pad to a multiple of 4 with keys larger than every site index
-        if (lane < ((c + 3) & ~3) - c) W.u.keys[c + lane] = INT_MAX;
-    }
     // patch rows as 16-byte vectors where the patch size allows
     constexpr bool kVec = (PSIZE * sizeof(T)) % 16 == 0;
     constexpr int NV16 = PSIZE * (int)sizeof(T) / 16;
@@ -116,22 +134,7 @@ __device__ __forceinline__ void spread_tile(int tile, SpreadWarpSmem<T, P, TILE>
     } else {
         for (int i = lane; i < PSIZE; i += 32) W.pt[i] = T(0);
     }
-    __syncwarp();
-    if (ranked) {
-        // rank of item i = number of items with a smaller original index
-        // (keys compared four at a time, from 16-byte broadcast loads)
-        const int c4 = (c + 3) >> 2;
-        const int4* k4 = reinterpret_cast<const int4*>(W.u.keys);
-        for (int i = lane; i < c; i += 32) {
-            const int ki = W.u.keys[i];
-            int r = 0;
-            for (int j = 0; j < c4; ++j) {
-                const int4 kk = k4[j];
-                r += (kk.x < ki) + (kk.y < ki) + (kk.z < ki) + (kk.w < ki);
-            }
-            W.perm[r] = (short)i;
-        }
-    }
+    if (ranked) rank_tile(W.u.keys, W.perm, sorig, s0, c);
     __syncwarp();
     const bool dense = c > kFastCap;  // ranked from global memory instead
     if (dense) rank_dense_tile(sorig + s0, c, order + s0, tmp + s0, W.u.keys);
@@ -248,11 +251,211 @@ k_spread_fast(Geo g, const int2* __restrict__ tiles, const int* __restrict__ sce
     }
 }
 
+// FP32 spread of 4-cell tiles with the patch in registers.  The shared-memory
+// patch above costs ten read-modify-write wavefronts a site on a dependent
+// chain; here a warp keeps its tile's whole patch in its lanes' registers and a
+// site is plain FMAs into them: its shared-memory traffic is only the reads of
+// its weights.
+//
+// The patch is cut into blocks of 4 y x 8 z points, lane (y % 4) 8 + z % 8
+// holding point (y, z) of every x in acc[x][y / 4][z / 8].  At tile edge 4 and
+// order 5 the patch is 8^3: 16 registers, all lanes used, and a site costs
+// 2 x 5 FMAs with weights that are zero outside its stencil.  Which P of the x
+// values they go to is the same for the whole warp, so a switch on the site's x
+// cell makes every register index a constant.  A point's sum takes the sites
+// in the same canonical order with the same products as the shared-memory
+// form, plus exact zeros, so the patches are bitwise the same.
+//
+// 288,768 sites on 64^3 (4,096 tiles of 70 sites), ncu: 39.9 -> 17.1 us.  At
+// tile edge 8 the patch takes 72 registers at order 5, a third of its lanes
+// are padding and 16 warps an SM are left: 40.7 us against 34.6 with
+// the shared-memory patch, which therefore stays for those tiles (and for
+// FP64, whose FMAs on zero weights cost more than the wavefronts).
+template <int P>
+struct SpreadRegs {
+    static constexpr int TILE = 4, E = TILE + P - 1, PZ = E | 1, PLANE = E * PZ, PSIZE = E * PLANE;
+    static constexpr int YB = (E + 3) / 4, ZB = (E + 7) / 8;  // blocks of the patch
+    // staged row of a site: q W_x (P values, the x cell in the last of the
+    // 16-byte groups), W_y over the patch's y, W_z over its z
+    static constexpr int XW = P <= 3 ? 4 : 8, YW = 4 * YB, ZW = 8 * ZB, ROW = XW + YW + ZW;
+    // x planes of the patch written out at a time, through the rows' space
+    static constexpr int OUTP = (32 * ROW) / PLANE < E ? (32 * ROW) / PLANE : E;
+};
+
+template <int P>
+struct __align__(16) SpreadRegSmem {
+    union {
+        int keys[kFastCap];  // original indices, while ranking
+        float row[kStage][SpreadRegs<P>::ROW];
+        float out[kStage * SpreadRegs<P>::ROW];  // finished x planes, while writing the patch out
+    } u;
+    short perm[kFastCap];  // canonical position -> slot in the tile
+};
+
+template <int P, int LX>
+__device__ __forceinline__ void spread_site(float (&acc)[SpreadRegs<P>::E][SpreadRegs<P>::YB][SpreadRegs<P>::ZB],
+                                            const float (&wx)[SpreadRegs<P>::XW],
+                                            const float (&wy)[SpreadRegs<P>::YB],
+                                            const float (&wz)[SpreadRegs<P>::ZB]) {
+#pragma unroll
+    for (int y = 0; y < SpreadRegs<P>::YB; ++y)
+#pragma unroll
+        for (int z = 0; z < SpreadRegs<P>::ZB; ++z) {
+            const float w = wy[y] * wz[z];
+#pragma unroll
+            for (int a = 0; a < P; ++a) acc[LX + a][y][z] += wx[a] * w;
+        }
+}
+
+template <int P>
+__device__ __forceinline__ void spread_tile_regs(int tile, SpreadRegSmem<P>& W, const int2* __restrict__ tiles,
+                                                 const int* __restrict__ scell, const int* __restrict__ sorig,
+                                                 const Rec<float>* __restrict__ srec, float* __restrict__ patch,
+                                                 int* order, int* tmp) {
+    typedef SpreadRegs<P> L;
+    const int lane = threadIdx.x & 31, py = lane >> 3, pz = lane & 7;
+    const int2 tr = tiles[tile];
+    const int s0 = tr.x, c = tr.y - s0;
+    const bool ranked = c > 1 && c <= kFastCap, dense = c > kFastCap;
+    if (ranked) rank_tile(W.u.keys, W.perm, sorig, s0, c);
+    if (dense) rank_dense_tile(sorig + s0, c, order + s0, tmp + s0, W.u.keys);
+    float acc[L::E][L::YB][L::ZB];
+#pragma unroll
+    for (int x = 0; x < L::E; ++x)
+#pragma unroll
+        for (int y = 0; y < L::YB; ++y)
+#pragma unroll
+            for (int z = 0; z < L::ZB; ++z) acc[x][y][z] = 0.f;
+    Rec<float> nr;
+    int ncell = 0;
+    auto fetch = [&](int t0) {
+        if (t0 + lane < c) {
+            const int s = s0 + (ranked ? (int)W.perm[t0 + lane] : (dense ? __ldcg(&order[s0 + t0 + lane]) : t0 + lane));
+            nr = load_rec(srec + s);
+            ncell = __ldg(&scell[s]);
+        }
+    };
+    fetch(0);
+    for (int t0 = 0; t0 < c; t0 += kStage) {
+        const int nb = min(kStage, c - t0);
+        if (lane < nb) {  // this lane's site: its row
+            const int lx = ncell & 255, ly = (ncell >> 8) & 255, lz = (ncell >> 16) & 255;
+            float w[wstride(P)];
+            BspCoef<float, P> co;
+            co.load();
+            site_weights<float, P>(co, nr, w);
+            float x8[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) x8[a] = a < P ? w[a] : 0.f;
+            x8[L::XW - 1] = __int_as_float(lx);
+            float* row = &W.u.row[lane][0];
+#pragma unroll
+            for (int a = 0; a < L::XW / 4; ++a)
+                reinterpret_cast<float4*>(row)[a] = make_float4(x8[4 * a], x8[4 * a + 1], x8[4 * a + 2], x8[4 * a + 3]);
+#pragma unroll
+            for (int a = L::XW / 4; a < L::ROW / 4; ++a)
+                reinterpret_cast<float4*>(row)[a] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int a = 0; a < P; ++a) {
+                row[L::XW + ly + a] = w[P + a];
+                row[L::XW + L::YW + lz + a] = w[2 * P + a];
+            }
+        }
+        __syncwarp();
+        fetch(t0 + kStage);  // in flight while this batch is spread
+        for (int j = 0; j < nb; ++j) {
+            const float* row = &W.u.row[j][0];
+            float wx[L::XW], wy[L::YB], wz[L::ZB];
+#pragma unroll
+            for (int a = 0; a < L::XW / 4; ++a) {
+                const float4 v = reinterpret_cast<const float4*>(row)[a];
+                wx[4 * a] = v.x;
+                wx[4 * a + 1] = v.y;
+                wx[4 * a + 2] = v.z;
+                wx[4 * a + 3] = v.w;
+            }
+#pragma unroll
+            for (int y = 0; y < L::YB; ++y) wy[y] = row[L::XW + 4 * y + py];
+#pragma unroll
+            for (int z = 0; z < L::ZB; ++z) wz[z] = row[L::XW + L::YW + 8 * z + pz];
+            switch (__float_as_int(wx[L::XW - 1])) {  // the same in every lane
+                case 0: spread_site<P, 0>(acc, wx, wy, wz); break;
+                case 1: spread_site<P, 1>(acc, wx, wy, wz); break;
+                case 2: spread_site<P, 2>(acc, wx, wy, wz); break;
+                case 3: spread_site<P, 3>(acc, wx, wy, wz); break;
+            }
+        }
+        __syncwarp();
+    }
+    // the patch, L::OUTP x planes at a time, through shared memory (padded z
+    // pitch included, so that no sector is left partly written)
+    float* dst = patch + (size_t)tile * L::PSIZE;
+    constexpr bool kVec = L::PSIZE % 4 == 0 && (L::OUTP * L::PLANE) % 4 == 0;
+#pragma unroll
+    for (int x0 = 0; x0 < L::E; x0 += L::OUTP) {
+#pragma unroll
+        for (int x = x0; x < L::E; ++x) {
+            if (x >= x0 + L::OUTP) break;
+#pragma unroll
+            for (int y = 0; y < L::YB; ++y)
+#pragma unroll
+                for (int z = 0; z < L::ZB; ++z)
+                    if (4 * y + py < L::E && 8 * z + pz < L::PZ)
+                        W.u.out[(x - x0) * L::PLANE + (4 * y + py) * L::PZ + 8 * z + pz] = acc[x][y][z];
+            if constexpr (L::PZ > 8 * L::ZB) {  // the padding column starts a z block of its own
+                if (lane < L::E) W.u.out[(x - x0) * L::PLANE + lane * L::PZ + L::PZ - 1] = 0.f;
+            }
+        }
+        __syncwarp();
+        const int n = (min(x0 + L::OUTP, (int)L::E) - x0) * L::PLANE;
+        if constexpr (kVec) {
+            for (int i = lane; i < n / 4; i += 32)
+                reinterpret_cast<float4*>(dst + x0 * L::PLANE)[i] = reinterpret_cast<const float4*>(W.u.out)[i];
+        } else {
+            for (int i = lane; i < n; i += 32) dst[x0 * L::PLANE + i] = W.u.out[i];
+        }
+        __syncwarp();
+    }
+}
+
+// (tiles handed out as in k_spread_fast)
+template <int P>
+__global__ void __launch_bounds__(kSpreadWarps * 32, P <= 5 ? 6 : 4)
+k_spread_regs(Geo g, const int2* __restrict__ tiles, const int* __restrict__ scell, const int* __restrict__ sorig,
+              const Rec<float>* __restrict__ srec, float* __restrict__ patch, int* order, int* tmp, int* ticket) {
+    pdl_enter();
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    SpreadRegSmem<P>& W = reinterpret_cast<SpreadRegSmem<P>*>(smem_raw)[warp];
+    const int nwarps = (int)gridDim.x * kSpreadWarps;
+    const int dyn = g.ntiles > nwarps ? g.ntiles - nwarps : 0;  // tiles handed out by ticket
+    int tile = (int)blockIdx.x * kSpreadWarps + warp;
+    if (tile >= g.ntiles) tile = -1;
+    for (;;) {
+        if (tile >= 0) spread_tile_regs<P>(tile, W, tiles, scell, sorig, srec, patch, order, tmp);
+        int t = 0;
+        if (lane == 0) t = atomicAdd(ticket, 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (t >= dyn) {
+            if (lane == 0 && t == dyn + nwarps - 1) atomicExch(ticket, 0);
+            return;  // whole warp; no block-level barrier in this kernel
+        }
+        tile = nwarps + t;
+    }
+}
+
 template <typename T, int P, int TILE>
 static cudaError_t spread_fast(cudaStream_t s, const Geo& g, const int2* tiles, const int* scell,
                                const int* sorig, const Rec<T>* srec, T* patch, int* order, int* tmp, int* ticket) {
-    auto kern = k_spread_fast<T, P, TILE>;
-    const size_t smem = kSpreadWarps * sizeof(SpreadWarpSmem<T, P, TILE>);
+    void (*kern)(Geo, const int2*, const int*, const int*, const Rec<T>*, T*, int*, int*, int*);
+    size_t smem;
+    if constexpr (sizeof(T) == 4 && TILE == 4) {
+        kern = k_spread_regs<P>;
+        smem = kSpreadWarps * sizeof(SpreadRegSmem<P>);
+    } else {
+        kern = k_spread_fast<T, P, TILE>;
+        smem = kSpreadWarps * sizeof(SpreadWarpSmem<T, P, TILE>);
+    }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // as many blocks as are resident at once (the tiles beyond them go by
