@@ -153,7 +153,8 @@ int setup_tiles(pppm_plan* P, int T) {
     dfree(P->patch);
     dfree(P->cov_off);
     dfree(P->cov_ent);
-    dfree(P->cov2);
+    dfree(P->cov_x);
+    dfree(P->cov_yz);
     dfree(P->tile_count);
     dfree(P->tiles);
     dfree(P->region_flag);
@@ -198,21 +199,34 @@ int setup_tiles(pppm_plan* P, int T) {
     if ((rc = dalloc(&P->cov_ent, sizeof(int2) * ent.size())) != PPPM_OK) return rc;
     CK(cudaMemcpy(P->cov_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(P->cov_ent, ent.data(), sizeof(int2) * ent.size(), cudaMemcpyHostToDevice));
-    // the same lists in two-slot form, if no index has more than two covers
+    // the same lists as the forward z FFT reads them, up to four a mesh index
     {
-        std::vector<int4> c2(3 * (size_t)nmax, make_int4(-1, 0, -1, 0));
-        bool ok = true;
+        std::vector<int2> cx(4 * (size_t)nmax, make_int2(-1, 0));
+        std::vector<int4> cyz(2 * (size_t)nmax, make_int4(-1, -1, -1, -1));
+        // (more than two covers everywhere, tile edge 4 with orders 6 and 7: the
+        // fold kernel and a mesh between are faster, 21.4 against 30.5 us on 64^3)
+        bool ok = p - 1 <= T;
+        P->cov_deep = false;
         for (int d = 0; d < 3 && ok; ++d)
             for (int m = 0; m < g.N[d]; ++m) {
                 const int b = off[(size_t)d * nmax1 + m], e = off[(size_t)d * nmax1 + m + 1];
-                if (e - b > 2) { ok = false; break; }
-                int4& v = c2[(size_t)d * nmax + m];
-                if (e - b >= 1) { v.x = ent[b].x; v.y = ent[b].y; }
-                if (e - b == 2) { v.z = ent[b + 1].x; v.w = ent[b + 1].y; }
+                if (e - b > 4) { ok = false; break; }
+                if (e - b > 2) P->cov_deep = true;
+                for (int k = b; k < e; ++k) {
+                    if (d == 0) {
+                        cx[4 * (size_t)m + (k - b)] = ent[k];
+                        continue;
+                    }
+                    int4& v = cyz[(d == 1 ? 0 : (size_t)nmax) + m];
+                    int* slot = k - b == 0 ? &v.x : k - b == 1 ? &v.y : k - b == 2 ? &v.z : &v.w;
+                    *slot = d == 1 ? ent[k].x * g.nt[2] * (int)psz + ent[k].y * g.Pz : ent[k].x * (int)psz + ent[k].y;
+                }
             }
         if (ok) {
-            if ((rc = dalloc(&P->cov2, sizeof(int4) * c2.size())) != PPPM_OK) return rc;
-            CK(cudaMemcpy(P->cov2, c2.data(), sizeof(int4) * c2.size(), cudaMemcpyHostToDevice));
+            if ((rc = dalloc(&P->cov_x, sizeof(int2) * cx.size())) != PPPM_OK) return rc;
+            if ((rc = dalloc(&P->cov_yz, sizeof(int4) * cyz.size())) != PPPM_OK) return rc;
+            CK(cudaMemcpy(P->cov_x, cx.data(), sizeof(int2) * cx.size(), cudaMemcpyHostToDevice));
+            CK(cudaMemcpy(P->cov_yz, cyz.data(), sizeof(int4) * cyz.size(), cudaMemcpyHostToDevice));
         }
     }
     P->tileT = T;
@@ -344,12 +358,14 @@ PatchSrc<T> patch_source(const pppm_plan* P) {
     const Geo& g = P->g;
     PatchSrc<T> ps{};
     ps.patch = (const T*)P->patch;
-    ps.cov2 = P->cov2;
+    ps.cov = P->cov_x;
+    ps.off = P->cov_yz;
+    ps.deep = P->cov_deep;
     int nmax = g.N[0];
     if (g.N[1] > nmax) nmax = g.N[1];
     if (g.N[2] > nmax) nmax = g.N[2];
     ps.nmax = nmax;
-    ps.psz = g.E[0] * g.E[1] * g.Pz;
+    ps.xstride = (int64_t)g.nt[1] * g.nt[2] * g.E[0] * g.E[1] * g.Pz;
     return ps;
 }
 
@@ -365,15 +381,17 @@ int run_solve(pppm_plan* P, cudaStream_t s, double* energy, double* virial, T* f
     C* c1 = (C*)P->cx[1];
     C* c2 = (C*)P->cx[2];
     { PROF(K_FFT_Z_R2C);
-      if (P->cov2)
+      if (P->cov_x)
           CK(launch_fft_z_r2c<T>(s, g, P->rad[2], (const C*)P->tw[2], nullptr, c0, patch_source<T>(P)));
       else
           CK(launch_fft_z_r2c<T>(s, g, P->rad[2], (const C*)P->tw[2], (const T*)P->rho, c0, PatchSrc<T>{})); }
     { PROF(K_FFT_Y); CK(launch_fft_bundle<T>(s, g, 1, -1, P->rad[1], P->lb[LB_Y], (const C*)P->tw[1], c0)); }
     { PROF(K_FFT_X_INFLUENCE);
       CK(launch_fft_x_influence<T>(s, g, P->rad[0], P->lb[LB_X_INFLUENCE], (const C*)P->tw[0], (const T*)P->G, P->beta, e_scale,
-                                   c_field, c0, c1, (T*)P->partial, P->counter, P->opt.prefactor, energy, virial)); }
-    { PROF(K_FFT_Y_INV3); CK(launch_fft_y_inverse3<T>(s, g, P->rad[1], P->lb[LB_Y_INVERSE3], (const C*)P->tw[1], c0, c1, c2)); }
+                                   c_field, c0, c1, (T*)P->partial)); }
+    { PROF(K_FFT_Y_INV3); CK(launch_fft_y_inverse3<T>(s, g, P->rad[1], P->lb[LB_Y_INVERSE3], (const C*)P->tw[1], c0, c1, c2,
+                                  (const T*)P->partial, x_influence_blocks(P->lb[LB_X_INFLUENCE]), P->opt.prefactor,
+                                  energy, virial)); }
     const int64_t N3 = mesh_points(P);
     const C* src[4] = {c1, c2, c0, c0};
     const int mk[4] = {0, 0, 1, 0};
@@ -402,8 +420,8 @@ int run_compute(pppm_plan* P, cudaStream_t s, const In* pos, const In* q, int64_
     // the kernels of the sequence overlap their launches (not under per-kernel
     // event timing, whose events must bracket each kernel)
     PdlScope pdl(P->pdl && !P->prof_on);
-    // with a two-slot cover table the forward z FFT folds the patches itself
-    T* rho = P->cov2 ? (T*)nullptr : (T*)P->rho;
+    // with the fold tables the forward z FFT folds the patches itself
+    T* rho = P->cov_x ? (T*)nullptr : (T*)P->rho;
     if ((rc = run_sites_to_patches<T, In>(P, s, pos, q, n, rho, T(1))) != PPPM_OK) return rc;
     T* fl = fields_out ? fields_out : (T*)P->fields;
     if ((rc = run_solve<T>(P, s, energy, virial, fl)) != PPPM_OK) return rc;
@@ -620,9 +638,7 @@ int pppm_create(const double box[3], const int mesh[3], int order, double beta, 
     }
     const int nblk = x_influence_blocks(P->lb[LB_X_INFLUENCE]);
     if ((rc = dalloc(&P->partial, 14 * P->esz * (size_t)nblk)) != PPPM_OK) return fail(rc);
-    if ((rc = dalloc(&P->counter, sizeof(unsigned int))) != PPPM_OK) return fail(rc);
     if ((rc = dalloc(&P->status, sizeof(int))) != PPPM_OK) return fail(rc);
-    if (cudaMemset(P->counter, 0, sizeof(unsigned int)) != cudaSuccess) return fail(PPPM_ERR_CUDA);
     if (cudaMemset(P->status, 0, sizeof(int)) != cudaSuccess) return fail(PPPM_ERR_CUDA);
     for (int d = 0; d < 3; ++d) {
         cudaError_t e = precision == PPPM_FP32 ? launch_twiddles<float>(P->own, mesh[d], (float2*)P->tw[d])
@@ -676,12 +692,12 @@ void pppm_destroy(pppm_plan* P) {
     for (int c = 0; c < 3; ++c) dfree(P->cx[c]);
     dfree(P->fields);
     dfree(P->partial);
-    dfree(P->counter);
     dfree(P->status);
     dfree(P->patch);
     dfree(P->cov_off);
     dfree(P->cov_ent);
-    dfree(P->cov2);
+    dfree(P->cov_x);
+    dfree(P->cov_yz);
     dfree(P->tile_count);
     dfree(P->tiles);
     dfree(P->region_flag);

@@ -17,33 +17,18 @@
 // Twiddles come from a table of e^{-2 pi i t / L} built on the device in FP64
 // with sincospi and rounded to the mesh precision.
 //
-// Two FFT engines drive the same kernels: CtEngine<L> for the common FP32 mesh
-// lengths (32 to 256: every index and radix is a compile-time constant), and
-// GenEngine for any other 2^a 3^b 5^c length and for FP64 (radix plan read at
-// run time).
-#include <type_traits>
-
-#include "fft_common.cuh"
+// The kernels here serve any 2^a 3^b 5^c length (radix plan read at run time);
+// lengths up to 256 (FP64: 128) run the same passes on the register engines
+// instead (fft_reg.cuh, fft_xy.cuh, fft_z.cuh), a line's points in registers
+// with every index and radix a compile-time constant.
+#include "fft_xy.cuh"
 #include "internal.cuh"
 
 namespace pppm {
 
-template <typename R, int L>
-struct CtEngine {
-    typedef typename CT<R>::C C;
-    static constexpr int kLen = L;  // compile-time length (0: known at run time)
-    const C* tw;
-    __device__ __forceinline__ static constexpr int len() { return L; }
-    template <int SIGN, bool LF>
-    __device__ __forceinline__ C* run(C* a, C* b, int nl, int ls, int ps) const {
-        return ct_fft<R, L, SIGN, LF, 0>(a, b, nl, ls, ps, tw);
-    }
-};
-
 template <typename R>
 struct GenEngine {
     typedef typename CT<R>::C C;
-    static constexpr int kLen = 0;
     Radix rp;
     const C* tw;
     __device__ __forceinline__ int len() const { return rp.L; }
@@ -52,32 +37,6 @@ struct GenEngine {
         return stockham<R>(a, b, nl, ls, ps, rp, tw, R(SIGN), LF);
     }
 };
-
-// Runs f(engine) with the compile-time engine when one exists for (T, L).
-template <typename T, typename F>
-cudaError_t with_engine(const Radix& r, const typename Cx<T>::t* tw, F&& f) {
-    if constexpr (std::is_same<T, float>::value) {
-        switch (r.L) {
-            case 32: return f(CtEngine<float, 32>{tw});
-            case 48: return f(CtEngine<float, 48>{tw});
-            case 64: return f(CtEngine<float, 64>{tw});
-            case 72: return f(CtEngine<float, 72>{tw});
-            case 80: return f(CtEngine<float, 80>{tw});
-            case 90: return f(CtEngine<float, 90>{tw});
-            case 96: return f(CtEngine<float, 96>{tw});
-            case 100: return f(CtEngine<float, 100>{tw});
-            case 108: return f(CtEngine<float, 108>{tw});
-            case 120: return f(CtEngine<float, 120>{tw});
-            case 128: return f(CtEngine<float, 128>{tw});
-            case 144: return f(CtEngine<float, 144>{tw});
-            case 160: return f(CtEngine<float, 160>{tw});
-            case 192: return f(CtEngine<float, 192>{tw});
-            case 256: return f(CtEngine<float, 256>{tw});
-            default: break;
-        }
-    }
-    return f(GenEngine<T>{r, tw});
-}
 
 template <typename K>
 cudaError_t set_smem(K kernel, size_t smem) {
@@ -100,32 +59,29 @@ cudaError_t set_smem(K kernel, size_t smem) {
 
 // ------------------------------------------------------------------ z forward (R2C)
 // Sum of the tile patches covering mesh point (x, y, z) (the fold of the
-// atomics-free spread) in a fixed order: the two x slots, two y slots and two
-// z slots give at most eight independent loads, empty slots contributing 0.
+// atomics-free spread) in a fixed order.
 template <typename R>
-__device__ __forceinline__ R fold_point(const Geo& g, const PatchSrc<R>& ps, int4 cx, int4 cy, int z) {
-    const int4 cz = __ldg(&ps.cov2[2 * ps.nmax + z]);
-    const int tx[2] = {cx.x, cx.z}, ox[2] = {cx.y, cx.w};
-    const int ty[2] = {cy.x, cy.z}, oy[2] = {cy.y, cy.w};
-    const int tz[2] = {cz.x, cz.z}, oz[2] = {cz.y, cz.w};
+__device__ __forceinline__ R fold_point(const Geo& g, const PatchSrc<R>& ps, int x, int y, int z) {
+    const int4 oy = __ldg(&ps.off[y]), oz = __ldg(&ps.off[ps.nmax + z]);
+    const int y4[4] = {oy.x, oy.y, oy.z, oy.w}, z4[4] = {oz.x, oz.y, oz.z, oz.w};
     R sum = R(0);
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < 4; ++a) {
+        const int2 cx = __ldg(&ps.cov[4 * x + a]);
+        if (cx.x < 0) break;
+        const R* px = ps.patch + (int64_t)cx.x * ps.xstride + cx.y * (g.E[1] * g.Pz);
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
+        for (int b = 0; b < 4; ++b)
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                if (tx[a] >= 0 && ty[b] >= 0 && tz[c] >= 0) {
-                    const int tile = (tx[a] * g.nt[1] + ty[b]) * g.nt[2] + tz[c];
-                    sum += ps.patch[(size_t)tile * ps.psz + (ox[a] * g.E[1] + oy[b]) * g.Pz + oz[c]];
-                }
-            }
+            for (int c = 0; c < 4; ++c)
+                if (y4[b] >= 0 && z4[c] >= 0) sum += px[y4[b] + z4[c]];
+    }
     return sum;
 }
 
-template <typename R, typename Eng>
+template <typename R>
 __global__ void __launch_bounds__(kFftThreads)
-k_fft_z_r2c(Geo g, Eng eng, const R* __restrict__ in, typename CT<R>::C* __restrict__ out, int rows, int pairs,
+k_fft_z_r2c(Geo g, GenEngine<R> eng, const R* __restrict__ in, typename CT<R>::C* __restrict__ out, int rows, int pairs,
             PatchSrc<R> ps) {
     pdl_enter();
     typedef typename CT<R>::C C;
@@ -140,21 +96,13 @@ k_fft_z_r2c(Geo g, Eng eng, const R* __restrict__ in, typename CT<R>::C* __restr
     const int npairs_total = (rows + 1) / 2;
     const int np = min(pairs, npairs_total - pair0);
     if (ps.patch) {
-        const int4 empty = make_int4(-1, 0, -1, 0);
         for (int p = threadIdx.x >> 5; p < np; p += kFftThreads >> 5) {
             const int r0 = 2 * (pair0 + p), r1 = r0 + 1;
             const int x0 = r0 / g.N[1], y0 = r0 - x0 * g.N[1];
-            const int4 cx0 = __ldg(&ps.cov2[x0]), cy0 = __ldg(&ps.cov2[ps.nmax + y0]);
-            int4 cx1 = empty, cy1 = empty;
-            if (r1 < rows) {
-                const int x1 = r1 / g.N[1], y1 = r1 - x1 * g.N[1];
-                cx1 = __ldg(&ps.cov2[x1]);
-                cy1 = __ldg(&ps.cov2[ps.nmax + y1]);
-            }
-#pragma unroll 2
+            const int x1 = r1 / g.N[1], y1 = r1 - x1 * g.N[1];
             for (int t = threadIdx.x & 31; t < Nz; t += 32) {
-                const R va = fold_point(g, ps, cx0, cy0, t);
-                const R vb = fold_point(g, ps, cx1, cy1, t);  // empty slots give 0
+                const R va = fold_point(g, ps, x0, y0, t);
+                const R vb = r1 < rows ? fold_point(g, ps, x1, y1, t) : R(0);
                 a[t * PL + p] = CT<R>::mk(va, vb);
             }
         }
@@ -182,6 +130,8 @@ k_fft_z_r2c(Geo g, Eng eng, const R* __restrict__ in, typename CT<R>::C* __restr
 template <typename T>
 cudaError_t launch_fft_z_r2c(cudaStream_t s, const Geo& g, const Radix& rz, const typename Cx<T>::t* tw,
                              const T* in, typename Cx<T>::t* out, const PatchSrc<T>& ps) {
+    const cudaError_t re = reg_z_r2c<T>(s, g, tw, in, out, ps);
+    if (re != cudaErrorNotSupported) return re;
     const int rows = g.N[0] * g.N[1];
     // up to 15 row pairs (an odd count) per block, within 32 KB of shared memory
     int pairs = (int)((32 * 1024) / (2 * g.N[2] * sizeof(typename Cx<T>::t)));
@@ -189,22 +139,20 @@ cudaError_t launch_fft_z_r2c(cudaStream_t s, const Geo& g, const Radix& rz, cons
     pairs |= 1;
     const int npairs = (rows + 1) / 2;
     const size_t smem = 2ull * pairs * g.N[2] * sizeof(typename Cx<T>::t);
-    return with_engine<T>(rz, tw, [&](auto eng) {
-        auto kern = k_fft_z_r2c<T, decltype(eng)>;
-        cudaError_t e = set_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-        return launch_k(kern, dim3((npairs + pairs - 1) / pairs), dim3(kFftThreads), smem, s, g, eng, in, out, rows,
-                        pairs, ps);
-    });
+    auto kern = k_fft_z_r2c<T>;
+    cudaError_t e = set_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    return launch_k(kern, dim3((npairs + pairs - 1) / pairs), dim3(kFftThreads), smem, s, g, GenEngine<T>{rz, tw}, in,
+                    out, rows, pairs, ps);
 }
 
 // ------------------------------------------------------------------ strided-line C2C
 // axis 1: lines along y (outer index x); axis 0: lines along x (outer index y).
 // Four resident blocks (64 registers): with the lines per block chosen for it,
 // the strided passes run in one round of blocks at the workload sizes.
-template <typename R, typename Eng, int SIGN>
+template <typename R, int SIGN>
 __global__ void __launch_bounds__(kFftThreads, 4)
-k_fft_bundle(Geo g, int axis, LineBlocks lb, Eng eng, typename CT<R>::C* __restrict__ data) {
+k_fft_bundle(Geo g, int axis, LineBlocks lb, GenEngine<R> eng, typename CT<R>::C* __restrict__ data) {
     pdl_enter();
     typedef typename CT<R>::C C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -234,13 +182,13 @@ k_fft_bundle(Geo g, int axis, LineBlocks lb, Eng eng, typename CT<R>::C* __restr
 template <typename T>
 cudaError_t launch_fft_bundle(cudaStream_t s, const Geo& g, int axis, int sign, const Radix& r, const LineBlocks& lb,
                               const typename Cx<T>::t* tw, typename Cx<T>::t* data) {
+    const cudaError_t re = reg_lines<T>(s, g, axis, sign, lb, tw, data);
+    if (re != cudaErrorNotSupported) return re;
     const size_t smem = 2ull * r.L * lb.B * sizeof(typename Cx<T>::t);
-    return with_engine<T>(r, tw, [&](auto eng) {
-        auto kern = sign < 0 ? k_fft_bundle<T, decltype(eng), -1> : k_fft_bundle<T, decltype(eng), 1>;
-        cudaError_t e = set_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-        return launch_k(kern, dim3(lb.nblk), dim3(kFftThreads), smem, s, g, axis, lb, eng, data);
-    });
+    auto kern = sign < 0 ? k_fft_bundle<T, -1> : k_fft_bundle<T, 1>;
+    cudaError_t e = set_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    return launch_k(kern, dim3(lb.nblk), dim3(kFftThreads), smem, s, g, axis, lb, GenEngine<T>{r, tw}, data);
 }
 
 // a / b for the virial coefficient: in FP32 the 2-ulp hardware quotient (the
@@ -259,7 +207,7 @@ __device__ __forceinline__ double div_approx(double a, double b) { return a / b;
 //      compensated (TwoSum) pairs;
 //   3. P = G rho_hat / (N h^3) and -i kx' P (kx' = 0 on the Nyquist index);
 //   4. inverse FFT along x of both; P -> S (in place), -i kx' P -> Bx.
-// The last block to finish sums the per-block partials (TwoSum in the mesh
+// A block of the y inverse sums the per-block partials (TwoSum in the mesh
 // precision, hi + lo in FP64 at the end) in a fixed order.
 //
 // Half-spectrum weights: w = 1 on the kz = 0 plane (and kz = Nz/2 for even Nz),
@@ -267,27 +215,14 @@ __device__ __forceinline__ double div_approx(double a, double b) { return a / b;
 // mirrored mode whose x (or y) index is the Nyquist index keeps that component's
 // sign (the index maps to itself, m = +N/2), so a product k_a k_b survives the
 // pairing only when both or neither of its components flip sign.
-// (h, l) += (h2, l2) with the rounding error of h + h2 carried into l
 template <typename R>
-__device__ __forceinline__ void two_sum_pair(R& h, R& l, R h2, R l2) {
-    R s = h + h2;
-    R bp = s - h;
-    R err = (h - (s - bp)) + (h2 - bp);
-    h = s;
-    l = l + l2 + err;
-}
-
-template <typename R, typename Eng>
 __global__ void __launch_bounds__(kFftThreads, 4)
-k_fft_x_influence(Geo g, LineBlocks lb, Eng eng, const R* __restrict__ G, R beta, R e_scale, R c_field,
-                  typename CT<R>::C* __restrict__ S, typename CT<R>::C* __restrict__ Bx, R* __restrict__ partial,
-                  unsigned int* __restrict__ counter, double prefactor, double* __restrict__ energy,
-                  double* __restrict__ virial) {
+k_fft_x_influence(Geo g, LineBlocks lb, GenEngine<R> eng, const R* __restrict__ G, R beta, R e_scale, R c_field,
+                  typename CT<R>::C* __restrict__ S, typename CT<R>::C* __restrict__ Bx, R* __restrict__ partial) {
     pdl_enter();
     typedef typename CT<R>::C C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ R red[kFftThreads / 32][14];
-    __shared__ bool is_last;
     const int Nx = eng.len(), Ny = g.N[1], Nz = g.N[2], Hz = g.Hz, B = lb.B;
     // lines along x, numbered f = y Hz + kz: a block's B lines are consecutive in memory
     const int64_t es = (int64_t)Ny * Hz;
@@ -302,18 +237,6 @@ k_fft_x_influence(Geo g, LineBlocks lb, Eng eng, const R* __restrict__ G, R beta
     C* b0 = a1 + Nx * B;
     C* base = S + f0;
     BUNDLE_LOOP(t, l, Nx, nl) a0[t * B + l] = base[t * es + l];
-    // with a compile-time length of whole 16-row passes, each thread's G values
-    // are fetched now so that their latency hides behind the forward FFT
-    constexpr bool kPre = Eng::kLen > 0 && Eng::kLen % (kFftThreads / 16) == 0;
-    constexpr int NG = kPre ? Eng::kLen / (kFftThreads / 16) : 1;
-    R gpre[NG];
-    if constexpr (kPre) {
-#pragma unroll
-        for (int i = 0; i < NG; ++i) {
-            const int t = (threadIdx.x >> 4) + i * (kFftThreads / 16);
-            gpre[i] = lt < nl ? __ldg(&G[(int64_t)t * es + f0 + lt]) : R(0);
-        }
-    }
     __syncthreads();
     C* rh = eng.template run<-1, true>(a0, a1, nl, 1, B);
     C* pbuf = (rh == a0) ? a1 : a0;  // free partner of the result buffer
@@ -355,13 +278,8 @@ k_fft_x_influence(Geo g, LineBlocks lb, Eng eng, const R* __restrict__ G, R beta
         b0[t * B + lt] = CT<R>::mk(kxd * P.y, -kxd * P.x);  // -i kx' P
     };
     if (lt < nl) {
-        if constexpr (kPre) {
-#pragma unroll
-            for (int i = 0; i < NG; ++i) mode((threadIdx.x >> 4) + i * (kFftThreads / 16), gpre[i]);
-        } else {
 #pragma unroll 1
-            for (int t = threadIdx.x >> 4; t < Nx; t += kFftThreads >> 4) mode(t, G[(int64_t)t * es + f0 + lt]);
-        }
+        for (int t = threadIdx.x >> 4; t < Nx; t += kFftThreads >> 4) mode(t, G[(int64_t)t * es + f0 + lt]);
     }
     __syncthreads();
     C* rA = eng.template run<1, true>(pbuf, rh, nl, 1, B);  // rho_hat is no longer needed: scratch
@@ -393,35 +311,6 @@ k_fft_x_influence(Geo g, LineBlocks lb, Eng eng, const R* __restrict__ G, R beta
         partial[(int64_t)blockIdx.x * 14 + 2 * q] = h;
         partial[(int64_t)blockIdx.x * 14 + 2 * q + 1] = lo;
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned int done = atomicAdd(counter, 1u);
-        is_last = (done == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (is_last) {
-        __threadfence();
-        if (warp < 7) {  // warp q sums quantity q over all blocks, then the FP64 final sum
-            const int q = warp;
-            R h = R(0), lo = R(0);
-            for (unsigned int b = lane; b < gridDim.x; b += 32) {
-                two_sum_pair(h, lo, __ldcg(&partial[(int64_t)b * 14 + 2 * q]),
-                             __ldcg(&partial[(int64_t)b * 14 + 2 * q + 1]));
-            }
-            for (int off = 16; off > 0; off >>= 1) {
-                const R h2 = __shfl_down_sync(0xffffffffu, h, off);
-                const R l2 = __shfl_down_sync(0xffffffffu, lo, off);
-                two_sum_pair(h, lo, h2, l2);
-            }
-            if (lane == 0) {
-                const double sum = ((double)h + (double)lo) * prefactor;
-                if (q == 0) energy[0] = sum;
-                else virial[q - 1] = sum;
-            }
-        }
-        if (threadIdx.x == 0) *counter = 0u;
-    }
 }
 
 int x_influence_blocks(const LineBlocks& lb) { return lb.nblk; }
@@ -429,30 +318,35 @@ int x_influence_blocks(const LineBlocks& lb) { return lb.nblk; }
 template <typename T>
 cudaError_t launch_fft_x_influence(cudaStream_t s, const Geo& g, const Radix& rx, const LineBlocks& lb,
                                    const typename Cx<T>::t* tw, const T* G, double beta, double e_scale,
-                                   double c_field, typename Cx<T>::t* S, typename Cx<T>::t* Bx, T* partial,
-                                   unsigned int* counter, double prefactor, double* energy, double* virial) {
+                                   double c_field, typename Cx<T>::t* S, typename Cx<T>::t* Bx, T* partial) {
+    const cudaError_t re = reg_x_influence<T>(s, g, lb, tw, G, beta, e_scale, c_field, S, Bx, partial);
+    if (re != cudaErrorNotSupported) return re;
     const size_t smem = 3ull * g.N[0] * lb.B * sizeof(typename Cx<T>::t);
-    return with_engine<T>(rx, tw, [&](auto eng) {
-        auto kern = k_fft_x_influence<T, decltype(eng)>;
-        cudaError_t e = set_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-        return launch_k(kern, dim3(x_influence_blocks(lb)), dim3(kFftThreads), smem, s, g, lb, eng, G, (T)beta,
-                        (T)e_scale, (T)c_field, S, Bx, partial, counter, prefactor, energy, virial);
-    });
+    auto kern = k_fft_x_influence<T>;
+    cudaError_t e = set_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    return launch_k(kern, dim3(x_influence_blocks(lb)), dim3(kFftThreads), smem, s, g, lb, GenEngine<T>{rx, tw}, G,
+                    (T)beta, (T)e_scale, (T)c_field, S, Bx, partial);
 }
 
 // ------------------------------------------------------------------ y inverse, three outputs
-// C = IFFT_y(A), D = IFFT_y(-i ky' A), Ex' = IFFT_y(Bx); C overwrites A, Ex' overwrites Bx.
-template <typename R, typename Eng>
+// C = IFFT_y(A), D = IFFT_y(-i ky' A), Ex' = IFFT_y(Bx); C overwrites A, Ex'
+// overwrites Bx.  Block 0 sums the x pass's energy partials beside the others.
+template <typename R>
 __global__ void __launch_bounds__(kFftThreads, 4)
-k_fft_y_inverse3(Geo g, LineBlocks lb, Eng eng, typename CT<R>::C* __restrict__ A, typename CT<R>::C* __restrict__ Bx,
-                 typename CT<R>::C* __restrict__ D) {
+k_fft_y_inverse3(Geo g, LineBlocks lb, GenEngine<R> eng, typename CT<R>::C* __restrict__ A, typename CT<R>::C* __restrict__ Bx,
+                 typename CT<R>::C* __restrict__ D, const R* __restrict__ partial, int npart, double prefactor,
+                 double* __restrict__ energy, double* __restrict__ virial) {
     pdl_enter();
+    if (blockIdx.x == 0) {
+        finish_energy(partial, npart, prefactor, energy, virial);
+        return;
+    }
     typedef typename CT<R>::C C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Ny = eng.len(), Hz = g.Hz, B = lb.B;
     // lines along y, numbered f = x Hz + kz; line f starts at x Ny Hz + kz
-    const int64_t f0 = (int64_t)blockIdx.x * B;
+    const int64_t f0 = (int64_t)(blockIdx.x - 1) * B;
     const int nl = (int)min((int64_t)B, (int64_t)g.N[0] * Hz - f0);
     const int64_t fl = f0 + (threadIdx.x & 15);  // this thread's line (B <= 16)
     const int64_t loff = (fl / Hz) * ((int64_t)Ny * Hz) + fl % Hz;
@@ -487,35 +381,22 @@ k_fft_y_inverse3(Geo g, LineBlocks lb, Eng eng, typename CT<R>::C* __restrict__ 
 template <typename T>
 cudaError_t launch_fft_y_inverse3(cudaStream_t s, const Geo& g, const Radix& ry, const LineBlocks& lb,
                                   const typename Cx<T>::t* tw, typename Cx<T>::t* A, typename Cx<T>::t* Bx,
-                                  typename Cx<T>::t* D) {
+                                  typename Cx<T>::t* D, const T* partial, int npart, double prefactor,
+                                  double* energy, double* virial) {
+    const cudaError_t re = reg_y_inverse3<T>(s, g, lb, tw, A, Bx, D, partial, npart, prefactor, energy, virial);
+    if (re != cudaErrorNotSupported) return re;
     const size_t smem = 4ull * g.N[1] * lb.B * sizeof(typename Cx<T>::t);
-    return with_engine<T>(ry, tw, [&](auto eng) {
-        auto kern = k_fft_y_inverse3<T, decltype(eng)>;
-        cudaError_t e = set_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-        return launch_k(kern, dim3(lb.nblk), dim3(kFftThreads), smem, s, g, lb, eng, A, Bx, D);
-    });
+    auto kern = k_fft_y_inverse3<T>;
+    cudaError_t e = set_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    return launch_k(kern, dim3(lb.nblk + 1), dim3(kFftThreads), smem, s, g, lb, GenEngine<T>{ry, tw}, A, Bx, D,
+                    partial, npart, prefactor, energy, virial);
 }
 
 // ------------------------------------------------------------------ z inverse (C2R)
-struct ZOut {
-    const void* src[4];
-    void* out[4];
-    int mulkz[4];
-    int nf;
-    FieldLayout fl;
-};
-
-// element f of a 4-entry kernel-parameter array, by selects (a dynamic index
-// would copy the whole parameter struct to local memory)
-template <typename X>
-__device__ __forceinline__ X pick4(const X (&a)[4], int f) {
-    return f == 0 ? a[0] : f == 1 ? a[1] : f == 2 ? a[2] : a[3];
-}
-
-template <typename R, typename Eng>
+template <typename R>
 __global__ void __launch_bounds__(kFftThreads, 6)  // six resident blocks: two rounds instead of three
-k_fft_z_c2r(Geo g, Eng eng, ZOut zo, int rows, int pairs) {
+k_fft_z_c2r(Geo g, GenEngine<R> eng, ZOut zo, int rows, int pairs) {
     pdl_enter();
     typedef typename CT<R>::C C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -628,6 +509,8 @@ cudaError_t launch_fft_z_c2r(cudaStream_t s, const Geo& g, const Radix& rz, cons
         zo.out[f] = f < nf ? out[f] : nullptr;
         zo.mulkz[f] = f < nf ? mulkz[f] : 0;
     }
+    const cudaError_t re = reg_z_c2r<T>(s, g, tw, zo);
+    if (re != cudaErrorNotSupported) return re;
     const int rows = g.N[0] * g.N[1];
     // at most 16 lines (nf fields x pairs) per block, the 16 lanes of a group
     // each taking one line in the FFT stages
@@ -635,35 +518,24 @@ cudaError_t launch_fft_z_c2r(cudaStream_t s, const Geo& g, const Radix& rz, cons
     if (pairs < 1) pairs = 1;
     const int npairs = (rows + 1) / 2;
     const size_t smem = 2ull * ((nf * pairs) | 1) * g.N[2] * sizeof(typename Cx<T>::t);
-    return with_engine<T>(rz, tw, [&](auto eng) {
-        auto kern = k_fft_z_c2r<T, decltype(eng)>;
-        cudaError_t e = set_smem(kern, smem);
-        if (e != cudaSuccess) return e;
-        return launch_k(kern, dim3((npairs + pairs - 1) / pairs), dim3(kFftThreads), smem, s, g, eng, zo, rows, pairs);
-    });
+    auto kern = k_fft_z_c2r<T>;
+    cudaError_t e = set_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    return launch_k(kern, dim3((npairs + pairs - 1) / pairs), dim3(kFftThreads), smem, s, g, GenEngine<T>{rz, tw}, zo,
+                    rows, pairs);
 }
 
 // B for one pass: the fewest rounds of resident blocks, then the fewest
 // blocks on the busiest SM (a block costs about the same for any B <= 16:
-// its lanes are laid out for 16 lines), then the larger B.
-template <typename K>
-static LineBlocks pick_line_blocks(K kern, size_t bytes_per_line, int64_t lines, int nsm) {
-    int maxB = 16;
-    while (maxB > 1 && bytes_per_line * maxB > 227 * 1024) --maxB;
+// its lanes are laid out for 16 lines), then the larger B.  resident(B) gives
+// the resident blocks per SM.
+template <typename F>
+static LineBlocks pick_line_blocks(F resident, int maxB, int64_t lines, int nsm) {
     LineBlocks best{1, (int)lines};
     int64_t best_rounds = -1, best_busy = 0;
-    if (set_smem(kern, bytes_per_line * maxB) != cudaSuccess) {
-        cudaGetLastError();
-        return best;
-    }
     for (int B = 1; B <= maxB; ++B) {
-        int per = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kFftThreads, bytes_per_line * B) !=
-                cudaSuccess ||
-            per < 1) {
-            cudaGetLastError();
-            continue;
-        }
+        const int per = resident(B);
+        if (per < 1) continue;
         const int64_t blocks = (lines + B - 1) / B;
         const int64_t rounds = (blocks + (int64_t)per * nsm - 1) / ((int64_t)per * nsm);
         const int64_t busy = (blocks + nsm - 1) / nsm;
@@ -676,23 +548,38 @@ static LineBlocks pick_line_blocks(K kern, size_t bytes_per_line, int64_t lines,
     return best;
 }
 
+template <typename T, typename K>
+static LineBlocks pass_line_blocks(int pass, K kern, int nbuf, int L, int64_t lines, int nsm) {
+    const int reg = reg_resident<T>(pass, L);
+    if (reg > 0) return pick_line_blocks([&](int) { return reg; }, 16, lines, nsm);
+    const size_t per_line = nbuf * sizeof(typename Cx<T>::t) * L;
+    int maxB = 16;
+    while (maxB > 1 && per_line * maxB > 227 * 1024) --maxB;
+    if (set_smem(kern, per_line * maxB) != cudaSuccess) {
+        cudaGetLastError();
+        return LineBlocks{1, (int)lines};
+    }
+    return pick_line_blocks(
+        [&](int B) {
+            int per = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kFftThreads, per_line * B) != cudaSuccess) {
+                cudaGetLastError();
+                return 0;
+            }
+            return per;
+        },
+        maxB, lines, nsm);
+}
+
 template <typename T>
 cudaError_t choose_line_blocks(const Geo& g, const Radix rad[3], int nsm, LineBlocks lb[4]) {
-    typedef typename Cx<T>::t C;
     const int64_t Hz = g.Hz;
-    cudaError_t e = with_engine<T>(rad[1], nullptr, [&](auto eng) {
-        lb[LB_Y] = pick_line_blocks(k_fft_bundle<T, decltype(eng), -1>, 2 * sizeof(C) * rad[1].L, g.N[0] * Hz, nsm);
-        lb[LB_Y_INVERSE3] =
-            pick_line_blocks(k_fft_y_inverse3<T, decltype(eng)>, 4 * sizeof(C) * rad[1].L, g.N[0] * Hz, nsm);
-        return cudaSuccess;
-    });
-    if (e != cudaSuccess) return e;
-    return with_engine<T>(rad[0], nullptr, [&](auto eng) {
-        lb[LB_X_INFLUENCE] =
-            pick_line_blocks(k_fft_x_influence<T, decltype(eng)>, 3 * sizeof(C) * rad[0].L, g.N[1] * Hz, nsm);
-        lb[LB_X] = pick_line_blocks(k_fft_bundle<T, decltype(eng), 1>, 2 * sizeof(C) * rad[0].L, g.N[1] * Hz, nsm);
-        return cudaSuccess;
-    });
+    const int Lx = rad[0].L, Ly = rad[1].L;
+    lb[LB_Y] = pass_line_blocks<T>(LB_Y, k_fft_bundle<T, -1>, 2, Ly, g.N[0] * Hz, nsm);
+    lb[LB_Y_INVERSE3] = pass_line_blocks<T>(LB_Y_INVERSE3, k_fft_y_inverse3<T>, 4, Ly, g.N[0] * Hz, nsm);
+    lb[LB_X_INFLUENCE] = pass_line_blocks<T>(LB_X_INFLUENCE, k_fft_x_influence<T>, 3, Lx, g.N[1] * Hz, nsm);
+    lb[LB_X] = pass_line_blocks<T>(LB_X, k_fft_bundle<T, 1>, 2, Lx, g.N[1] * Hz, nsm);
+    return cudaSuccess;
 }
 
 #define PPPM_INST_FFT(T)                                                                                           \
@@ -703,9 +590,10 @@ cudaError_t choose_line_blocks(const Geo& g, const Radix rad[3], int nsm, LineBl
                                               const Cx<T>::t*, Cx<T>::t*);                                         \
     template cudaError_t launch_fft_x_influence<T>(cudaStream_t, const Geo&, const Radix&, const LineBlocks&,      \
                                                    const Cx<T>::t*, const T*, double, double, double, Cx<T>::t*,   \
-                                                   Cx<T>::t*, T*, unsigned int*, double, double*, double*);        \
+                                                   Cx<T>::t*, T*);                                                 \
     template cudaError_t launch_fft_y_inverse3<T>(cudaStream_t, const Geo&, const Radix&, const LineBlocks&,       \
-                                                  const Cx<T>::t*, Cx<T>::t*, Cx<T>::t*, Cx<T>::t*);               \
+                                                  const Cx<T>::t*, Cx<T>::t*, Cx<T>::t*, Cx<T>::t*, const T*, int, \
+                                                  double, double*, double*);                                       \
     template cudaError_t launch_fft_z_c2r<T>(cudaStream_t, const Geo&, const Radix&, const Cx<T>::t*, int,         \
                                              const Cx<T>::t* const*, const int*, T* const*, const FieldLayout&);
 PPPM_INST_FFT(float)

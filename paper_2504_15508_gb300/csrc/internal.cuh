@@ -56,16 +56,20 @@ struct Geo {
 };
 
 // Where the forward z FFT reads its real input: a mesh, or the spread's tile
-// patches summed on the fly (the fold), through the per-axis cover lists.
-// Each mesh index is covered by at most two tile patches per axis when every
-// axis holds at least T + p - 1 points; cov2[d * nmax + m] lists them as
-// {tile, coordinate, tile, coordinate}, tile -1 for an empty slot.
+// patches summed on the fly (the fold), through the per-axis cover lists: the
+// (tile, patch coordinate) pairs covering each mesh index, in tile order.  The
+// tables hold up to four a mesh index: two where every tile is whole, three or
+// four near the seam of a mesh whose last tile is ragged.  The x entries
+// are {tile, coordinate}, the y and z entries offsets into the patches
+// (tile part + coordinate part), -1 where there is none.
 template <typename R>
 struct PatchSrc {
-    const R* patch;       // nullptr: read the mesh
-    const int4* cov2;     // two-slot cover table, 3 axes of nmax entries each
+    const R* patch;    // nullptr: read the mesh
+    const int2* cov;   // x: 4 entries a mesh index
+    const int4* off;   // y: off[m], z: off[nmax + m]
     int nmax;
-    int psz;              // elements per tile patch = E0 * E1 * Pz
+    int deep;          // some index has more than two covers
+    int64_t xstride;   // patch elements per x tile
 };
 
 template <typename R> __host__ __device__ __forceinline__ R kfac(const Geo& g, int d);
@@ -299,6 +303,22 @@ struct LineBlocks {
     int B;     // lines per block, at most 16
     int nblk;  // blocks = ceil(outer Hz / B)
 };
+// C2R outputs of the z inverse: nf fields (see launch_fft_z_c2r)
+struct ZOut {
+    const void* src[4];
+    void* out[4];
+    int mulkz[4];
+    int nf;
+    FieldLayout fl;
+};
+
+// element f of a 4-entry kernel-parameter array, by selects (a dynamic index
+// would copy the whole parameter struct to local memory)
+template <typename X>
+__device__ __forceinline__ X pick4(const X (&a)[4], int f) {
+    return f == 0 ? a[0] : f == 1 ? a[1] : f == 2 ? a[2] : a[3];
+}
+
 // the passes of a plan
 enum { LB_Y = 0, LB_X_INFLUENCE = 1, LB_Y_INVERSE3 = 2, LB_X = 3 };
 
@@ -379,15 +399,17 @@ cudaError_t launch_fft_z_r2c(cudaStream_t s, const Geo& g, const Radix& rz, cons
 template <typename T>
 cudaError_t launch_fft_bundle(cudaStream_t s, const Geo& g, int axis, int sign, const Radix& r, const LineBlocks& lb,
                               const typename Cx<T>::t* tw, typename Cx<T>::t* data);
+// x FFT, influence function, inverse x FFTs; the block's energy and virial sums
+// go to partial (14 values a block), which the y inverse adds up
 template <typename T>
 cudaError_t launch_fft_x_influence(cudaStream_t s, const Geo& g, const Radix& rx, const LineBlocks& lb,
                                    const typename Cx<T>::t* tw, const T* G, double beta, double e_scale,
-                                   double c_field, typename Cx<T>::t* S, typename Cx<T>::t* Bx, T* partial,
-                                   unsigned int* counter, double prefactor, double* energy, double* virial);
+                                   double c_field, typename Cx<T>::t* S, typename Cx<T>::t* Bx, T* partial);
 template <typename T>
 cudaError_t launch_fft_y_inverse3(cudaStream_t s, const Geo& g, const Radix& ry, const LineBlocks& lb,
                                   const typename Cx<T>::t* tw, typename Cx<T>::t* A, typename Cx<T>::t* Bx,
-                                  typename Cx<T>::t* D);
+                                  typename Cx<T>::t* D, const T* partial, int npart, double prefactor,
+                                  double* energy, double* virial);
 // nf fields: out[f] = C2R_z(src[f] * (mulkz[f] ? -i kz' : 1)); src/out arrays of nf pointers
 template <typename T>
 cudaError_t launch_fft_z_c2r(cudaStream_t s, const Geo& g, const Radix& rz, const typename Cx<T>::t* tw, int nf,
@@ -397,6 +419,28 @@ int x_influence_blocks(const LineBlocks& lb);
 // B of each pass (LB_*), from the resident blocks per SM of its kernel
 template <typename T>
 cudaError_t choose_line_blocks(const Geo& g, const Radix rad[3], int nsm, LineBlocks lb[4]);
+
+// fft_reg_*.cu: the passes on the register engines (cudaErrorNotSupported for a
+// length without one)
+template <typename T>
+cudaError_t reg_z_r2c(cudaStream_t s, const Geo& g, const typename Cx<T>::t* tw, const T* in,
+                      typename Cx<T>::t* out, const PatchSrc<T>& ps);
+template <typename T>
+cudaError_t reg_z_c2r(cudaStream_t s, const Geo& g, const typename Cx<T>::t* tw, const ZOut& zo);
+template <typename T>
+cudaError_t reg_lines(cudaStream_t s, const Geo& g, int axis, int sign, const LineBlocks& lb,
+                      const typename Cx<T>::t* tw, typename Cx<T>::t* data);
+template <typename T>
+cudaError_t reg_x_influence(cudaStream_t s, const Geo& g, const LineBlocks& lb, const typename Cx<T>::t* tw,
+                            const T* G, double beta, double e_scale, double c_field, typename Cx<T>::t* S,
+                            typename Cx<T>::t* Bx, T* partial);
+template <typename T>
+cudaError_t reg_y_inverse3(cudaStream_t s, const Geo& g, const LineBlocks& lb, const typename Cx<T>::t* tw,
+                           typename Cx<T>::t* A, typename Cx<T>::t* Bx, typename Cx<T>::t* D, const T* partial,
+                           int npart, double prefactor, double* energy, double* virial);
+// resident blocks per SM of a pass (LB_*) for lines of L points; 0: no engine
+template <typename T>
+int reg_resident(int pass, int L);
 
 // influence.cu
 cudaError_t launch_influence(cudaStream_t s, const Geo& g, double beta, int alias, double* G);

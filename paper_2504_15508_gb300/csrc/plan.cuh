@@ -35,14 +35,15 @@ struct pppm_plan {
     CUtensorMap fmap;        // 4D TMA descriptor of the padded fields
     bool fmap_ok = false;
     void* partial = nullptr;
-    unsigned int* counter = nullptr;
     int* status = nullptr;
     // tiles
     int tileT = 0;
     void* patch = nullptr;
     int* cov_off = nullptr;
     int2* cov_ent = nullptr;
-    int4* cov2 = nullptr;  // two-slot cover table (null when some index has more covers)
+    int2* cov_x = nullptr;  // fold tables of the forward z FFT (PatchSrc); null when
+    int4* cov_yz = nullptr; // some mesh index has more than four covers
+    bool cov_deep = false;
     int* tile_count = nullptr;
     int2* tiles = nullptr;     // per tile (first slot, end slot) of the tile-ordered site data
     int region_cap = 0;        // slots of a tile's fixed region (0: compact layout only)
