@@ -294,11 +294,10 @@ int pppm_set_potential(pppm_plan *plan, int on);
 /*
  * pppm_set_dependent_launch -- when on (nonzero, the default), the kernels of
  * one evaluation are launched with programmatic dependent launch: each may be
- * scheduled while its predecessor's last blocks run and waits on the device
- * for the predecessor to complete before touching memory.  That removes the
- * gaps between kernels of a plan running alone; when other work shares the
- * GPU concurrently (another stream), the early-scheduled blocks hold SM
- * resources that work could use, and off may overlap better.  Results are
+ * scheduled as soon as its predecessor's blocks have finished and waits on the
+ * device for the predecessor's writes before touching memory.  That shortens
+ * the gaps between kernels of a plan running alone; when other work shares the
+ * GPU concurrently (another stream), off may overlap better.  Results are
  * identical either way.  A graph captured before the change no longer
  * matches the plan (pppm_graph_launch refuses it).
  */

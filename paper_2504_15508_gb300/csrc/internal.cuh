@@ -94,16 +94,20 @@ struct FieldLayout {
 };
 
 // Programmatic dependent launch.  Within a plan's solve sequence each kernel
-// is launched with programmatic stream serialization: its blocks may be
-// scheduled while the previous kernel's last blocks still run, and it waits
+// is launched with programmatic stream serialization: it may be scheduled as
+// soon as the previous kernel's blocks have all finished, and waits
 // (griddepcontrol.wait, the first statement of every such kernel) until that
-// kernel has completed and its writes are visible before touching memory.
-// Each kernel also allows its successor to be scheduled as soon as all of its
-// own blocks have started.  Outside the sequence (or with per-kernel event
-// timing on) launches are plain; the wait is then a no-op.
+// kernel's writes are visible before touching memory, which hides most of the
+// gap between two launches.  No kernel triggers its successor earlier: blocks
+// scheduled while their predecessor still runs pile up on the SMs that have
+// room at that moment, and a grid of about one block an SM then finishes at
+// half the GPU (64^3 FP64: 241 us a step with the trigger at kernel start,
+// 168 without; 160^3: 205 and 193, 128^3: 149 and 143; the smallest box,
+// 32^3, the same 28.7).
+// Outside the sequence (or with per-kernel event timing on) launches are
+// plain; the wait is then a no-op.
 __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Canonical order of a tile that holds more sites than a spread kernel ranks
