@@ -27,77 +27,11 @@
 #include <new>
 #include <vector>
 
+#include "batched.cuh"
 #include "fft_common.cuh"
-#include "internal.cuh"
 
 namespace pppm {
 namespace batch {
-
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-enum Stage { S_BIN, S_SCAN, S_SCATTER, S_SPREAD, S_ZR2C, S_YFWD, S_XINF, S_YINV, S_ZC2R, S_GATHER, NSTAGE };
-constexpr int kSiteChunk = 1024;  // sites per bin / scatter item
-constexpr int kZPairs = 8;        // row pairs per z-pass item, at least
-constexpr int kZRows = 512;       // and up to about this many points (pairs x Nz) an item
-constexpr int kSpreadTiles = kWarps;
-constexpr int kGatherTiles = 2;   // four warps per tile
-
-struct BoxDesc {
-    Geo g;
-    Radix rad[3];
-    Bundle bd;
-    FieldLayout fl;
-    long long site0;
-    int nsite;
-    int tile0;   // into tile_count
-    int ts0;     // into tile_start (ntiles + 1 entries per box)
-    long long patch0;
-    long long c0;  // complex half-spectrum offset
-    long long f0;  // padded field offset (3 fields)
-    long long G0;
-    int tw0[3];
-    int cov0;
-    int nmax;
-    int part0;
-    float e_scale, c_field, beta;
-    int zp;  // row pairs per z-pass item
-    int nitems[NSTAGE];
-};
-
-struct Bufs {
-    const float* pos;
-    const float* q;
-    float* forces;
-    double* energy;
-    double* virial;
-    int* tile_count;
-    int* tile_start;
-    int* tile_of;
-    int* slot_of;
-    Rec<float>* rec;
-    int* cell;
-    int* scell;
-    int* sorig;
-    Rec<float>* srec;  // tile order: the sites' records (B-spline arguments, charge)
-    float* patch;
-    float2* cx0;
-    float2* cx1;
-    float2* cx2;
-    float* fields;
-    const float* G;
-    const float2* tw;
-    const int4* cov2;
-    float* partial;
-    unsigned int* box_counter;
-    int* box_fail;  // set when a wait of the box ran out: its later stages skip their work
-    int* status;
-    double prefactor;
-    int dft_max;  // lines up to this length take the tensor-core DFT (0: all take the FFT)
-    int qgroup;     // node size of the int32-quantised DFT (0: off)
-    double qscale;  // its scale
-    int wait_probe;  // 1: box 0's scan waits for one binning item more than exist (its wait runs out)
-    RedRows red_rows;  // lane -> stencil row of the spread's shared-memory atomics
-};
 
 // ------------------------------------------------------------------ helpers
 // All p B-spline weights N_p(x0 + j), j = 0..p-1, by the Cox-de Boor recursion
@@ -1102,9 +1036,17 @@ cudaError_t launch_one_stage(cudaStream_t s, const BoxDesc* boxes, const int2* i
     return launch_k(kern, dim3(count), dim3(kThreads), smem, s, boxes, items + start, B);
 }
 
+// The FFT stages of a staged launch on the register engines: their own items
+// (count 0: these meshes or options take the general stages).
+struct RegFft {
+    const int2* items = nullptr;
+    int start[NFFT + 1] = {};
+    size_t smem[NFFT] = {};
+};
+
 template <int P, int TILE, bool Q>
 cudaError_t launch_staged(cudaStream_t s, const BoxDesc* boxes, const int2* items, const int* stage_start,
-                          const Bufs& B, int maxN, int maxB, int maxZ) {
+                          const RegFft& reg, const Bufs& B, int maxN, int maxB, int maxZ) {
     PdlScope pdl(true);
     cudaError_t e = cudaSuccess;
 #define PPPM_STAGE(ST)                                                                                      \
@@ -1117,8 +1059,18 @@ cudaError_t launch_staged(cudaStream_t s, const BoxDesc* boxes, const int2* item
     e = launch_one_stage<5, 8, Q, ST>(s, boxes, items, stage_start[ST], stage_start[ST + 1] - stage_start[ST], \
                                       B, maxN, maxB, maxZ);                                                 \
     if (e != cudaSuccess) return e;
-    PPPM_STAGE(S_BIN) PPPM_STAGE(S_SCAN) PPPM_STAGE(S_SCATTER) PPPM_STAGE(S_SPREAD) PPPM_FFT_STAGE(S_ZR2C)
-    PPPM_FFT_STAGE(S_YFWD) PPPM_FFT_STAGE(S_XINF) PPPM_FFT_STAGE(S_YINV) PPPM_FFT_STAGE(S_ZC2R) PPPM_STAGE(S_GATHER)
+    PPPM_STAGE(S_BIN) PPPM_STAGE(S_SCAN) PPPM_STAGE(S_SCATTER) PPPM_STAGE(S_SPREAD)
+    if (reg.items) {
+        for (int k = 0; k < NFFT; ++k) {
+            e = launch_reg_fft(s, S_ZR2C + k, boxes, reg.items + reg.start[k], reg.start[k + 1] - reg.start[k], B,
+                               reg.smem[k]);
+            if (e != cudaSuccess) return e;
+        }
+    } else {
+        PPPM_FFT_STAGE(S_ZR2C) PPPM_FFT_STAGE(S_YFWD) PPPM_FFT_STAGE(S_XINF) PPPM_FFT_STAGE(S_YINV)
+        PPPM_FFT_STAGE(S_ZC2R)
+    }
+    PPPM_STAGE(S_GATHER)
 #undef PPPM_FFT_STAGE
 #undef PPPM_STAGE
     return e;
@@ -1163,6 +1115,10 @@ struct pppm_batch {
         BoxDesc* d_desc = nullptr;
         int2* d_items = nullptr;
         int4* d_cov2 = nullptr;
+        int2* d_cov_x = nullptr;   // fold tables of the register engines' z pass
+        int4* d_cov_yz = nullptr;
+        int2* d_ritems = nullptr;  // items of their FFT stages
+        RegFft reg;                // items null: some line has no engine
         int ntile_total = 0, ntile_start_total = 0;
         long long patch_total = 0;
         int part_total = 0;
@@ -1279,10 +1235,16 @@ int build_layout(pppm_batch* P, int li, int T) {
     bfree(Y.d_desc);
     bfree(Y.d_items);
     bfree(Y.d_cov2);
+    bfree(Y.d_cov_x);
+    bfree(Y.d_cov_yz);
+    bfree(Y.d_ritems);
     Y = pppm_batch::Layout();
     Y.T = T;
     const int p = P->order;
     std::vector<int4> cov;
+    std::vector<int2> cov_x;
+    std::vector<int4> cov_yz;
+    bool reg = true;
     long long patch0 = 0, c0 = 0, f0 = 0;
     int tile0 = 0, ts0 = 0, part0 = 0;
     Y.desc.resize(P->nbox);
@@ -1348,6 +1310,27 @@ int build_layout(pppm_batch* P, int li, int T) {
                     else return PPPM_ERR_BAD_MESH;
                 }
             }
+        // the same covers as the register engines' fold reads them
+        const int psz = D.g.E[0] * D.g.E[1] * D.g.Pz;
+        D.cov_x0 = (int)cov_x.size();
+        D.cov_yz0 = (int)cov_yz.size();
+        D.xstride = (long long)D.g.nt[1] * D.g.nt[2] * psz;
+        D.cov_deep = 0;
+        for (int d = 0; d < 3; ++d) reg = reg && reg_fft_length(N[d]);
+        cov_x.resize(cov_x.size() + 4 * (size_t)maxN, make_int2(-1, 0));
+        cov_yz.resize(cov_yz.size() + 2 * (size_t)maxN, make_int4(-1, -1, -1, -1));
+        for (int d = 0; d < 3; ++d)
+            for (int m = 0; m < N[d]; ++m) {
+                const int4 v0 = cov[D.cov0 + 2 * ((size_t)d * maxN + m)], v1 = cov[D.cov0 + 2 * ((size_t)d * maxN + m) + 1];
+                const int t[4] = {v0.x, v0.z, v1.x, v1.z}, c[4] = {v0.y, v0.w, v1.y, v1.w};
+                if (t[2] >= 0) D.cov_deep = 1;
+                int o[4];
+                for (int k = 0; k < 4; ++k) {
+                    if (d == 0) cov_x[D.cov_x0 + 4 * (size_t)m + k] = make_int2(t[k], c[k]);
+                    o[k] = t[k] < 0 ? -1 : d == 1 ? t[k] * D.g.nt[2] * psz + c[k] * D.g.Pz : t[k] * psz + c[k];
+                }
+                if (d > 0) cov_yz[D.cov_yz0 + (d == 1 ? 0 : (size_t)maxN) + m] = make_int4(o[0], o[1], o[2], o[3]);
+            }
         // every stage waits only on the one before it, so no stage may be
         // empty: a box without sites still gets one (idle) binning and one
         // scatter item, or its spread would not wait for its scan
@@ -1366,7 +1349,8 @@ int build_layout(pppm_batch* P, int li, int T) {
         D.nitems[S_ZC2R] = D.nitems[S_ZR2C];
         D.nitems[S_GATHER] = (D.g.ntiles + kGatherTiles - 1) / kGatherTiles;
         D.part0 = part0;
-        part0 += D.nitems[S_XINF];
+        for (int k = 0; k < NFFT; ++k) D.rnitems[k] = reg ? reg_fft_items(S_ZR2C + k, N, D.g.Hz) : 0;
+        part0 += std::max(D.nitems[S_XINF], D.rnitems[S_XINF - S_ZR2C]);
     }
     // stage-major work list; bigger boxes first within a stage
     std::vector<int> order(P->nbox);
@@ -1378,6 +1362,17 @@ int build_layout(pppm_batch* P, int li, int T) {
             for (int i = 0; i < Y.desc[b].nitems[s]; ++i) Y.items.push_back(make_int2(b | (s << 16), i));
     }
     Y.stage_start[NSTAGE] = (int)Y.items.size();
+    std::vector<int2> ritems;
+    if (reg) {
+        for (int k = 0; k < NFFT; ++k) {
+            Y.reg.start[k] = (int)ritems.size();
+            for (int b : order) {
+                for (int i = 0; i < Y.desc[b].rnitems[k]; ++i) ritems.push_back(make_int2(b, i));
+                Y.reg.smem[k] = std::max(Y.reg.smem[k], reg_fft_smem(S_ZR2C + k, &P->meshes[3 * b]));
+            }
+        }
+        Y.reg.start[NFFT] = (int)ritems.size();
+    }
     Y.ntile_total = tile0;
     Y.ntile_start_total = ts0;
     Y.patch_total = patch0;
@@ -1391,6 +1386,15 @@ int build_layout(pppm_batch* P, int li, int T) {
     BK(cudaMemcpy(Y.d_desc, Y.desc.data(), sizeof(BoxDesc) * Y.desc.size(), cudaMemcpyHostToDevice));
     BK(cudaMemcpy(Y.d_items, Y.items.data(), sizeof(int2) * Y.items.size(), cudaMemcpyHostToDevice));
     BK(cudaMemcpy(Y.d_cov2, cov.data(), sizeof(int4) * cov.size(), cudaMemcpyHostToDevice));
+    if ((rc = balloc(&Y.d_cov_x, sizeof(int2) * cov_x.size())) != PPPM_OK) return rc;
+    if ((rc = balloc(&Y.d_cov_yz, sizeof(int4) * cov_yz.size())) != PPPM_OK) return rc;
+    BK(cudaMemcpy(Y.d_cov_x, cov_x.data(), sizeof(int2) * cov_x.size(), cudaMemcpyHostToDevice));
+    BK(cudaMemcpy(Y.d_cov_yz, cov_yz.data(), sizeof(int4) * cov_yz.size(), cudaMemcpyHostToDevice));
+    if (reg) {
+        if ((rc = balloc(&Y.d_ritems, sizeof(int2) * ritems.size())) != PPPM_OK) return rc;
+        BK(cudaMemcpy(Y.d_ritems, ritems.data(), sizeof(int2) * ritems.size(), cudaMemcpyHostToDevice));
+        Y.reg.items = Y.d_ritems;
+    }
     // grow the shared work buffers
     if (Y.patch_total > P->patch_cap) {
         bfree(P->patch);
@@ -1464,6 +1468,8 @@ int enqueue(pppm_batch* P, cudaStream_t s, int li, const float* pos, const float
     B.G = P->G;
     B.tw = P->tw;
     B.cov2 = Y.d_cov2;
+    B.cov_x = Y.d_cov_x;
+    B.cov_yz = Y.d_cov_yz;
     B.partial = P->partial;
     B.box_counter = P->box_counter;
     B.box_fail = P->box_fail;
@@ -1477,9 +1483,11 @@ int enqueue(pppm_batch* P, cudaStream_t s, int li, const float* pos, const float
     cudaError_t e = cudaErrorInvalidValue;
     const int n = (int)Y.items.size();
     const bool quant = P->quant_group > 0;
+    // the quantised and the tensor-core DFT are options of the general stages
+    const RegFft reg = quant || P->dft_max > 0 ? RegFft() : Y.reg;
 #define BATCH_CASE(PP, TT, QQ)                                                                                   \
     if (P->order == PP && Y.T == TT && quant == QQ)                                                              \
-        e = P->staged ? launch_staged<PP, TT, QQ>(s, Y.d_desc, Y.d_items, Y.stage_start, B, Y.maxN, Y.maxB,      \
+        e = P->staged ? launch_staged<PP, TT, QQ>(s, Y.d_desc, Y.d_items, Y.stage_start, reg, B, Y.maxN, Y.maxB, \
                                                   Y.maxZ)                                                          \
                       : launch<PP, TT, QQ>(s, Y.d_desc, Y.d_items, n, P->head, P->done, B, P->spin_limit, Y.maxN, \
                                            Y.maxB, Y.maxZ, &P->last_grid);
@@ -1780,6 +1788,9 @@ void pppm_batch_destroy(pppm_batch* P) {
         bfree(Y.d_desc);
         bfree(Y.d_items);
         bfree(Y.d_cov2);
+        bfree(Y.d_cov_x);
+        bfree(Y.d_cov_yz);
+        bfree(Y.d_ritems);
     }
     bfree(P->G);
     bfree(P->tw);

@@ -120,6 +120,49 @@ __device__ __forceinline__ void fold_row(const Geo& g, const PatchSrc<R>& ps, in
     }
 }
 
+// The transform of a pair's rows from the points each thread holds (v[q][n] =
+// point B n + j + T q, row 0 + i row 1), and the two half rows out to o0 and
+// o0 + Hz (the second if `two`).
+template <typename R, int L>
+__device__ __forceinline__ void z_forward(typename CT<R>::C (&v)[FacZ<L>::G1][FacZ<L>::A], bool on, bool two, int j,
+                                          typename CT<R>::C* sm, const typename CT<R>::C* __restrict__ tw,
+                                          typename CT<R>::C* __restrict__ o0) {
+    typedef PairEngine<R, L> E;
+    typedef typename CT<R>::C C;
+    constexpr int A = E::A, B = E::B, T = E::T, G1 = E::G1, Hz = L / 2 + 1;
+#pragma unroll
+    for (int q = 0; q < G1; ++q)
+        if (on && j + T * q < B) E::space_out(v[q], j + T * q, sm, tw);
+    E::sync();
+    if (!on || j >= E::T2) return;
+    const int kb1 = pair_k1<A>(j);
+    const bool bon = pair_on<A>(j);
+    C za[B], zb[B];
+    E::spec_in(za, j, sm);
+    if (bon) {
+        E::spec_in(zb, kb1, sm);
+    } else {
+#pragma unroll
+        for (int k = 0; k < B; ++k) zb[k] = za[k];
+    }
+    C* o1 = o0 + Hz;
+    auto put = [&](int k, C z, C mirror) {  // x0 = (Z + conj Z') / 2, x1 = (Z - conj Z') / 2i
+        const C zc = cconj(mirror), d = csub(z, zc);
+        o0[k] = cscale(cadd(z, zc), R(0.5));
+        if (two) o1[k] = CT<R>::mk(R(0.5) * d.y, R(-0.5) * d.x);
+    };
+#pragma unroll
+    for (int k = 0; k <= B / 2; ++k) {
+        // mirror of k1 + A k2: (A - k1) + A (B - 1 - k2), of A k2: A (B - k2)
+        const C ma0 = za[(B - k) % B], mb = zb[B - 1 - (k < B ? k : 0)], maj = za[B - 1 - (k < B ? k : 0)];
+        const int ka = j + A * k, kb = kb1 + A * k;
+        const C ma = j > 0 ? mb : ma0;
+        if (ka < Hz) put(ka, za[k % B], ma);
+        const C mbb = j > 0 ? maj : mb;
+        if (bon && kb < Hz) put(kb, zb[k % B], mbb);
+    }
+}
+
 template <typename R, int L, bool SPLIT>
 __global__ void __launch_bounds__((SPLIT ? 2 : 1) * FacZ<L>::T * FacZ<L>::NPMAX,
                                   SPLIT ? pass_blocks<R, 2 * FacZ<L>::T * FacZ<L>::NPMAX>(40 + 7 * FacZ<L>::G1 * FacZ<L>::A / 2)
@@ -188,38 +231,7 @@ k_fft_z_r2c_reg(Geo g, const typename CT<R>::C* __restrict__ tw, const R* __rest
         }
         E::sync();  // before the line takes the hand-over's space
     }
-#pragma unroll
-    for (int q = 0; q < G1; ++q)
-        if (on && j + T * q < B) E::space_out(v[q], j + T * q, sm, tw);
-    E::sync();
-    if (!on || j >= E::T2) return;
-    const int kb1 = pair_k1<A>(j);
-    const bool bon = pair_on<A>(j);
-    C za[B], zb[B];
-    E::spec_in(za, j, sm);
-    if (bon) {
-        E::spec_in(zb, kb1, sm);
-    } else {
-#pragma unroll
-        for (int k = 0; k < B; ++k) zb[k] = za[k];
-    }
-    C* o0 = out + (int64_t)r0 * Hz;
-    C* o1 = o0 + Hz;
-    auto put = [&](int k, C z, C mirror) {  // x0 = (Z + conj Z') / 2, x1 = (Z - conj Z') / 2i
-        const C zc = cconj(mirror), d = csub(z, zc);
-        o0[k] = cscale(cadd(z, zc), R(0.5));
-        if (two) o1[k] = CT<R>::mk(R(0.5) * d.y, R(-0.5) * d.x);
-    };
-#pragma unroll
-    for (int k = 0; k <= B / 2; ++k) {
-        // mirror of k1 + A k2: (A - k1) + A (B - 1 - k2), of A k2: A (B - k2)
-        const C ma0 = za[(B - k) % B], mb = zb[B - 1 - (k < B ? k : 0)], maj = za[B - 1 - (k < B ? k : 0)];
-        const int ka = j + A * k, kb = kb1 + A * k;
-        const C ma = j > 0 ? mb : ma0;
-        if (ka < Hz) put(ka, za[k % B], ma);
-        const C mbb = j > 0 ? maj : mb;
-        if (bon && kb < Hz) put(kb, zb[k % B], mbb);
-    }
+    z_forward<R, L>(v, on, two, j, sm, tw, out + (int64_t)r0 * Hz);
 }
 
 // ------------------------------------------------------------------ z inverse (C2R)
@@ -271,6 +283,32 @@ __device__ __forceinline__ void z_join(const Geo& g, const typename CT<R>::C* __
     }
     E::spec_out(za, j, sm, tw);
     if (bon) E::spec_out(zb, kb1, sm, tw);
+}
+
+// store(o) for the offset o of row r of the padded layout and of each of its
+// periodic images (at most one per axis: Xp < 2 Nx)
+template <typename F>
+__device__ __forceinline__ void row_images(const Geo& g, const FieldLayout& fl, int r, F store) {
+    const int Nx = g.N[0], Ny = g.N[1], kmin = g.kmin;
+    const int x = r / Ny, y = r - x * Ny;
+    const int px0 = x - kmin, py0 = y - kmin;
+    const int pxg = px0 + Nx < fl.Xp ? px0 + Nx : (px0 - Nx >= 0 ? px0 - Nx : -1);
+    const int pyg = py0 + Ny < fl.Yp ? py0 + Ny : (py0 - Ny >= 0 ? py0 - Ny : -1);
+#pragma unroll 1
+    for (int im = 0; im < 4; ++im) {
+        const int px = (im & 1) ? pxg : px0, py = (im & 2) ? pyg : py0;
+        if (px >= 0 && py >= 0) store(((int64_t)px * fl.Yp + py) * fl.Zp);
+    }
+}
+
+// Point B n + n2 of a line of L to out[o + its padded z] and to its z ghost (only
+// the first and last few points have one); n is a constant where it is called.
+template <int L, int B, typename V>
+__device__ __forceinline__ void put_point(V* out, int64_t o, int n, int n2, int kmin, int Zp, V val) {
+    const int pz = B * n + n2 - kmin;
+    out[o + pz] = val;
+    if (B * n < kMaxOrder && pz + L < Zp) out[o + pz + L] = val;
+    if (B * (n + 1) > L - kMaxOrder && pz >= L) out[o + pz - L] = val;
 }
 
 // One field (blockIdx.y) into an unpadded mesh, two rows a line.
@@ -368,50 +406,30 @@ k_fft_z_c2r_reg(Geo g, const typename CT<R>::C* __restrict__ tw, ZOut zo, int ro
     __syncthreads();
     if (!ron || set == 0) return;
     const FieldLayout& fl = zo.fl;
-    const int kmin = g.kmin, Nx = g.N[0], Ny = g.N[1];
-    // store(o) for the offset o of row r and of each of its periodic images
-    // (at most one per axis: Xp < 2 Nx)
-    auto images = [&](int r, auto store) {
-        const int x = r / Ny, y = r - x * Ny;
-        const int px0 = x - kmin, py0 = y - kmin;
-        const int pxg = px0 + Nx < fl.Xp ? px0 + Nx : (px0 - Nx >= 0 ? px0 - Nx : -1);
-        const int pyg = py0 + Ny < fl.Yp ? py0 + Ny : (py0 - Ny >= 0 ? py0 - Ny : -1);
-#pragma unroll 1
-        for (int im = 0; im < 4; ++im) {
-            const int px = (im & 1) ? pxg : px0, py = (im & 2) ? pyg : py0;
-            if (px >= 0 && py >= 0) store(((int64_t)px * fl.Yp + py) * fl.Zp);
-        }
-    };
-    // point B n + n2 of a line to out[o + its padded z] and its z ghost (only the
-    // first and last few points have one)
-    auto put = [&](auto* out, int64_t o, int n, int n2, auto val) {
-        const int pz = B * n + n2 - kmin;
-        out[o + pz] = val;
-        if (B * n < kMaxOrder && pz + L < fl.Zp) out[o + pz + L] = val;
-        if (B * (n + 1) > L - kMaxOrder && pz >= L) out[o + pz - L] = val;
-    };
     if (set == 3) {
         R* phi = reinterpret_cast<R*>(zo.out[3]);
 #pragma unroll 1
         for (int half = 0; half < (two ? 2 : 1); ++half)
-            images(2 * pair + half, [&](int64_t o) {
+            row_images(g, fl, 2 * pair + half, [&](int64_t o) {
 #pragma unroll
                 for (int q = 0; q < G1; ++q)
 #pragma unroll
                     for (int n = 0; n < A; ++n)
-                        if (j + T * q < B) put(phi, o, n, j + T * q, half ? v[q][n].y : v[q][n].x);
+                        if (j + T * q < B)
+                            put_point<L, B>(phi, o, n, j + T * q, g.kmin, fl.Zp, half ? v[q][n].y : v[q][n].x);
             });
         return;
     }
     V4* out = reinterpret_cast<V4*>(zo.out[0]);
     const R* ezr = ez + (set - 1) * L;
-    images(2 * pair + set - 1, [&](int64_t o) {
+    row_images(g, fl, 2 * pair + set - 1, [&](int64_t o) {
 #pragma unroll
         for (int q = 0; q < G1; ++q)
 #pragma unroll
             for (int n = 0; n < A; ++n)
                 if (j + T * q < B)
-                    put(out, o, n, j + T * q, CT<R>::mk4(v[q][n].x, v[q][n].y, ezr[B * n + j + T * q], R(0)));
+                    put_point<L, B>(out, o, n, j + T * q, g.kmin, fl.Zp,
+                                    CT<R>::mk4(v[q][n].x, v[q][n].y, ezr[B * n + j + T * q], R(0)));
     });
 }
 
