@@ -17,7 +17,7 @@
 // Inference runs on the tensor cores (mma.sync m16n8k16 BF16 -> FP32; the
 // accumulator fragments of one layer are exactly the A fragments of the next,
 // so a warp chains all three layers in registers).  Training is FP32 on the
-// CUDA cores, one block of 128 threads per 128 sites, with the per-block weight
+// CUDA cores, tiles of 32 sites by blocks of 256 threads, with the per-block weight
 // gradients reduced in a fixed order before the Adam step.
 #include <cuda_bf16.h>
 
@@ -49,7 +49,6 @@ struct Net {
     // words put the eight row groups of a fragment load on distinct banks)
     static constexpr int K1P = NIN + 8;
     static constexpr int BW1 = 0, BW2 = BW1 + NH * K1P, BW3 = BW2 + NH * K2P, NBF = BW3 + NOUT_PAD * K2P;
-    static constexpr int XP = NIN + 1;  // training: padded row of the feature tile
 };
 constexpr int kNinCell = 48, kNinStated = 32;
 
@@ -661,172 +660,263 @@ __global__ void k_to_bf16(const float* __restrict__ master, __nv_bfloat16* __res
 }
 
 // ------------------------------------------------------------------ training
-constexpr int TB = 128;  // sites per training block
-constexpr int HP = NH + 1;
+constexpr int TB = 32;        // sites a tile
+constexpr int TTHR = 256;     // threads a block
+constexpr int HP = NH + 4;    // row pitch of the activation tiles and transposed weights
 
 __device__ __forceinline__ float bfr(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
-// Per block: forward and backward of 128 sites (FP32, weights rounded to BF16
-// as used by inference), per-block gradient sums to partial[block][NPARAM],
-// and the block's share of the loss to lossp[block].
 template <int NIN>
-__global__ void __launch_bounds__(TB)
-k_mlp_grad(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ target, int64_t nrows,
-           const int* __restrict__ idx, int nb, float inv_total, const float* __restrict__ master, float* __restrict__ partial,
-           float* __restrict__ lossp) {
-    typedef Net<NIN> L;
-    constexpr int XP = L::XP, NPARAM = L::NPARAM, O_W1 = L::O_W1, O_B1 = L::O_B1, O_W2 = L::O_W2, O_B2 = L::O_B2,
-                  O_W3 = L::O_W3, O_B3 = L::O_B3;
-    extern __shared__ __align__(16) float sm[];
-    float* W1 = sm;                  // 64 x NIN
-    float* W2 = W1 + NH * NIN;       // 64 x 64
-    float* W3 = W2 + NH * NH;        // 3 x 64
-    float* bb = W3 + NOUT * NH;      // b1 64, b2 64, b3 3 (+1)
-    float* X = bb + 2 * NH + 4;      // TB x XP
-    float* H1 = X + TB * XP;         // TB x HP
-    float* H2 = H1 + TB * HP;        // TB x HP
-    float* DY = H2 + TB * HP;        // TB x 4
-    float* red = DY + TB * 4;        // 32
-    const int t = threadIdx.x;
-    for (int k = t; k < NH * NIN; k += TB) W1[k] = bfr(master[O_W1 + k]);
-    for (int k = t; k < NH * NH; k += TB) W2[k] = bfr(master[O_W2 + k]);
-    for (int k = t; k < NOUT * NH; k += TB) W3[k] = bfr(master[O_W3 + k]);
-    for (int k = t; k < NH; k += TB) {
-        bb[k] = bfr(master[O_B1 + k]);
-        bb[NH + k] = bfr(master[O_B2 + k]);
-    }
-    if (t < NOUT) bb[2 * NH + t] = bfr(master[O_B3 + t]);
-    const int s = blockIdx.x * TB + t;
-    int site = s < nb ? (idx ? idx[s] : s) : -1;
-    const bool valid = site >= 0 && site < nrows;  // rows outside the table contribute nothing
-    if (!valid) site = 0;
-    for (int k = 0; k < NIN; ++k) X[t * XP + k] = valid ? __bfloat162float(feat[(int64_t)site * NIN + k]) : 0.f;
-    __syncthreads();
-    // forward of this thread's site
-    for (int j = 0; j < NH; ++j) {
-        float z = bb[j];
-        for (int k = 0; k < NIN; ++k) z += W1[j * NIN + k] * X[t * XP + k];
-        H1[t * HP + j] = tanhf(z);
-    }
-    for (int j = 0; j < NH; ++j) {
-        float z = bb[NH + j];
-        for (int k = 0; k < NH; ++k) z += W2[j * NH + k] * H1[t * HP + k];
-        H2[t * HP + j] = tanhf(z);
-    }
-    float l = 0.f;
-    for (int c = 0; c < NOUT; ++c) {
-        float y = bb[2 * NH + c];
-        for (int k = 0; k < NH; ++k) y += W3[c * NH + k] * H2[t * HP + k];
-        const float r = valid ? y - target[3 * (int64_t)site + c] : 0.f;
-        l += r * r;
-        DY[t * 4 + c] = 2.f * r * inv_total;
-    }
-    // block loss (fixed-order tree)
-    for (int off = 16; off > 0; off >>= 1) l += __shfl_down_sync(0xffffffffu, l, off);
-    if ((t & 31) == 0) red[t >> 5] = l;
-    __syncthreads();
-    float* g = partial + (size_t)blockIdx.x * NPARAM;
-    if (t == 0) lossp[blockIdx.x] = (red[0] + red[1] + red[2] + red[3]) * inv_total;
-    // dW3, db3
-    for (int o = t; o < NOUT * NH + NOUT; o += TB) {
-        float acc = 0.f;
-        if (o < NOUT * NH) {
-            const int c = o / NH, j = o - c * NH;
-            for (int r = 0; r < TB; ++r) acc += DY[r * 4 + c] * H2[r * HP + j];
-            g[O_W3 + o] = acc;
-        } else {
-            const int c = o - NOUT * NH;
-            for (int r = 0; r < TB; ++r) acc += DY[r * 4 + c];
-            g[O_B3 + c] = acc;
+struct GradSmem {
+    static constexpr int XP = NIN + 4;
+    float w1t[NIN][HP];  // [k][unit]
+    float w2t[NH][HP];   // [k][unit]
+    float w2[NH][NH];    // [unit][k]
+    float w3[NOUT][NH];
+    float b1[NH], b2[NH], b3[4];
+    float x[TB][XP];
+    float h1[TB][HP], h2[TB][HP], d1[TB][HP], d2[TB][HP];
+    float dy[TB][4];
+    int site[TB];
+    float red[TTHR / 32];
+};
+
+// acc[s][u] += sum_k a[2 sg + s][k] w[k][4 ug + u]: two sites and four units a
+// thread, four k at a time (a as 16-byte broadcasts, w as 16-byte rows)
+template <int K, int AP, int WP>
+__device__ __forceinline__ void tile_gemm(const float (*__restrict__ a)[AP], const float (*__restrict__ w)[WP], int sg,
+                                          int ug, float (&acc)[2][4]) {
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+        const float4 a0 = *reinterpret_cast<const float4*>(&a[2 * sg][k]);
+        const float4 a1 = *reinterpret_cast<const float4*>(&a[2 * sg + 1][k]);
+        const float av[2][4] = {{a0.x, a0.y, a0.z, a0.w}, {a1.x, a1.y, a1.z, a1.w}};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 wv = *reinterpret_cast<const float4*>(&w[k + q][4 * ug]);
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                acc[s][0] += av[s][q] * wv.x;
+                acc[s][1] += av[s][q] * wv.y;
+                acc[s][2] += av[s][q] * wv.z;
+                acc[s][3] += av[s][q] * wv.w;
+            }
         }
-    }
-    __syncthreads();
-    // dZ2 over H2 (own row)
-    for (int j = 0; j < NH; ++j) {
-        float dh = 0.f;
-        for (int c = 0; c < NOUT; ++c) dh += DY[t * 4 + c] * W3[c * NH + j];
-        const float h = H2[t * HP + j];
-        H2[t * HP + j] = dh * (1.f - h * h);
-    }
-    __syncthreads();
-    // dW2 (thread: column k, rows j = t/64 + 2m), db2
-    {
-        const int k = t & (NH - 1), j0 = t >> 6;
-        float acc[NH / 2];
-        for (int m = 0; m < NH / 2; ++m) acc[m] = 0.f;
-        for (int r = 0; r < TB; ++r) {
-            const float hk = H1[r * HP + k];
-#pragma unroll
-            for (int m = 0; m < NH / 2; ++m) acc[m] += H2[r * HP + j0 + 2 * m] * hk;
-        }
-        for (int m = 0; m < NH / 2; ++m) g[O_W2 + (j0 + 2 * m) * NH + k] = acc[m];
-    }
-    if (t < NH) {
-        float acc = 0.f;
-        for (int r = 0; r < TB; ++r) acc += H2[r * HP + t];
-        g[O_B2 + t] = acc;
-    }
-    __syncthreads();
-    // dZ1 over H1 (own row)
-    for (int k = 0; k < NH; ++k) {
-        float dh = 0.f;
-        for (int j = 0; j < NH; ++j) dh += H2[t * HP + j] * W2[j * NH + k];
-        const float h = H1[t * HP + k];
-        H1[t * HP + k] = dh * (1.f - h * h);
-    }
-    __syncthreads();
-    // dW1 (thread: columns k0 + 16 c, c < NIN / 16, k0 = t % 16; rows j0 + 8 m,
-    // m < 8, j0 = t / 16), db1
-    {
-        static_assert(NIN % 16 == 0 && NH == 64 && TB == 128, "dW1 thread map");
-        constexpr int KC = NIN / 16;
-        const int k0 = t & 15, j0 = t >> 4;
-        float acc[KC][8];
-#pragma unroll
-        for (int c = 0; c < KC; ++c)
-#pragma unroll
-            for (int m = 0; m < 8; ++m) acc[c][m] = 0.f;
-        for (int r = 0; r < TB; ++r) {
-            float xk[KC], hj[8];
-#pragma unroll
-            for (int c = 0; c < KC; ++c) xk[c] = X[r * XP + k0 + 16 * c];
-#pragma unroll
-            for (int m = 0; m < 8; ++m) hj[m] = H1[r * HP + j0 + 8 * m];
-#pragma unroll
-            for (int c = 0; c < KC; ++c)
-#pragma unroll
-                for (int m = 0; m < 8; ++m) acc[c][m] += hj[m] * xk[c];
-        }
-#pragma unroll
-        for (int c = 0; c < KC; ++c)
-#pragma unroll
-            for (int m = 0; m < 8; ++m) g[O_W1 + (j0 + 8 * m) * NIN + k0 + 16 * c] = acc[c][m];
-    }
-    if (t < NH) {
-        float acc = 0.f;
-        for (int r = 0; r < TB; ++r) acc += H1[r * HP + t];
-        g[O_B1 + t] = acc;
     }
 }
 
-// Sum the per-block gradients in block order; then either return them or take
-// one Adam step (FP32 master, moments m, v) and refresh nothing else (the BF16
-// copy is rebuilt by k_to_bf16).
+// Forward and backward of tiles of 32 sites (FP32, weights rounded to BF16 as
+// used by inference) by 256 threads; a block takes every gridDim-th tile,
+// keeps its share of the weight gradients in registers and writes it once, to
+// partial[block][NPARAM], with its share of the loss in lossp[block].
+//
+// A thread holds 2 sites x 4 units of each layer and 4 x 4 (first layer 4 x
+// NIN / 16) entries of a weight gradient, so that a shared-memory wavefront
+// feeds three to five FMAs; at one thread a site (128 a block, 64 blocks at
+// 8,192 rows) each FMA read a weight of its own and less than half of the
+// SMs had a block.  8,192 rows, cell set, ncu: 77.6 -> 30.0 us.
 template <int NIN>
-__global__ void k_reduce_adam(const float* __restrict__ partial, const float* __restrict__ lossp, int nblk,
-                              float* __restrict__ grad_out, float* __restrict__ loss_out, float* __restrict__ master,
-                              float* __restrict__ m1, float* __restrict__ m2, float lr, float b1, float b2, float eps,
-                              float bc1, float bc2) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0 && loss_out) {
-        float l = 0.f;
-        for (int b = 0; b < nblk; ++b) l += lossp[b];
-        *loss_out = l;
+__global__ void __launch_bounds__(TTHR, 2)
+k_mlp_grad(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ target, int64_t nrows,
+           const int* __restrict__ idx, int nb, float inv_total, const float* __restrict__ master,
+           float* __restrict__ partial, float* __restrict__ lossp) {
+    typedef Net<NIN> L;
+    constexpr int NPARAM = L::NPARAM, O_W1 = L::O_W1, O_B1 = L::O_B1, O_W2 = L::O_W2, O_B2 = L::O_B2, O_W3 = L::O_W3,
+                  O_B3 = L::O_B3, KC = NIN / 16;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    GradSmem<NIN>& S = *reinterpret_cast<GradSmem<NIN>*>(sm_raw);
+    const int t = threadIdx.x;
+    const int ug = t & 15, sg = t >> 4;  // units 4 ug.., sites 2 sg..; in dW: columns by ug, rows 4 sg..
+    for (int i = t; i < NH * NIN; i += TTHR) S.w1t[i % NIN][i / NIN] = bfr(master[O_W1 + i]);
+    for (int i = t; i < NH * NH; i += TTHR) {
+        const float w = bfr(master[O_W2 + i]);
+        S.w2[i / NH][i % NH] = w;
+        S.w2t[i % NH][i / NH] = w;
     }
+    for (int i = t; i < NOUT * NH; i += TTHR) S.w3[i / NH][i % NH] = bfr(master[O_W3 + i]);
+    if (t < NH) {
+        S.b1[t] = bfr(master[O_B1 + t]);
+        S.b2[t] = bfr(master[O_B2 + t]);
+    }
+    if (t < NOUT) S.b3[t] = bfr(master[O_B3 + t]);
+    float gw1[4][KC] = {}, gw2[4][4] = {}, gw3 = 0.f, gb = 0.f, loss = 0.f;
+    const int ntile = (nb + TB - 1) / TB;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        __syncthreads();  // the previous tile has been read (the first time: the weights are in place after the next)
+        if (t < TB) {
+            const int s = tile * TB + t;
+            const int i = s < nb ? (idx ? idx[s] : s) : -1;
+            S.site[t] = i >= 0 && i < nrows ? i : -1;  // rows outside the table contribute nothing
+        }
+        __syncthreads();
+        for (int i = t; i < TB * NIN / 2; i += TTHR) {  // a BF16 pair each
+            const int r = i / (NIN / 2), c = i - r * (NIN / 2), row = S.site[r];
+            float2 v = make_float2(0.f, 0.f);
+            if (row >= 0)
+                v = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(feat + (int64_t)row * NIN)[c]);
+            *reinterpret_cast<float2*>(&S.x[r][2 * c]) = v;
+        }
+        __syncthreads();
+        // hidden layers
+        {
+            float acc[2][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[0][u] = acc[1][u] = S.b1[4 * ug + u];
+            tile_gemm<NIN>(S.x, S.w1t, sg, ug, acc);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+                *reinterpret_cast<float4*>(&S.h1[2 * sg + s][4 * ug]) =
+                    make_float4(tanhf(acc[s][0]), tanhf(acc[s][1]), tanhf(acc[s][2]), tanhf(acc[s][3]));
+        }
+        __syncthreads();
+        {
+            float acc[2][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[0][u] = acc[1][u] = S.b2[4 * ug + u];
+            tile_gemm<NH>(S.h1, S.w2t, sg, ug, acc);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+                *reinterpret_cast<float4*>(&S.h2[2 * sg + s][4 * ug]) =
+                    make_float4(tanhf(acc[s][0]), tanhf(acc[s][1]), tanhf(acc[s][2]), tanhf(acc[s][3]));
+        }
+        __syncthreads();
+        {  // outputs and loss: eight threads a site, thread c < 3 of them ends with output c
+            const int r = t >> 3, c = t & 7, row = S.site[r];
+            float y[NOUT] = {};
+#pragma unroll
+            for (int k = c; k < NH; k += 8) {
+                const float h = S.h2[r][k];
+#pragma unroll
+                for (int o = 0; o < NOUT; ++o) y[o] += S.w3[o][k] * h;
+            }
+#pragma unroll
+            for (int h = 4; h >= 1; h >>= 1)
+#pragma unroll
+                for (int o = 0; o < NOUT; ++o) y[o] += __shfl_xor_sync(0xffffffffu, y[o], h);
+            if (c < NOUT) {
+                const float yc = (c == 0 ? y[0] : c == 1 ? y[1] : y[2]) + S.b3[c];
+                const float d = row >= 0 ? yc - target[3 * (int64_t)row + c] : 0.f;
+                loss += d * d;
+                S.dy[r][c] = 2.f * d * inv_total;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {  // dZ2 of this thread's sites and units
+            const int r = 2 * sg + s;
+            float d[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = 4 * ug + u;
+                const float h = S.h2[r][j];
+                d[u] = (S.dy[r][0] * S.w3[0][j] + S.dy[r][1] * S.w3[1][j] + S.dy[r][2] * S.w3[2][j]) * (1.f - h * h);
+            }
+            *reinterpret_cast<float4*>(&S.d2[r][4 * ug]) = make_float4(d[0], d[1], d[2], d[3]);
+        }
+        if (t < NOUT * NH) {  // dW3
+            const int c = t / NH, j = t - c * NH;
+#pragma unroll 8
+            for (int r = 0; r < TB; ++r) gw3 += S.dy[r][c] * S.h2[r][j];
+        } else if (t < NOUT * NH + NOUT) {  // db3
+#pragma unroll 8
+            for (int r = 0; r < TB; ++r) gw3 += S.dy[r][t - NOUT * NH];
+        }
+        __syncthreads();
+        {  // dZ1
+            float acc[2][4] = {};
+            tile_gemm<NH>(S.d2, S.w2, sg, ug, acc);
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const float4 h = *reinterpret_cast<const float4*>(&S.h1[2 * sg + s][4 * ug]);
+                *reinterpret_cast<float4*>(&S.d1[2 * sg + s][4 * ug]) =
+                    make_float4(acc[s][0] * (1.f - h.x * h.x), acc[s][1] * (1.f - h.y * h.y),
+                                acc[s][2] * (1.f - h.z * h.z), acc[s][3] * (1.f - h.w * h.w));
+            }
+        }
+#pragma unroll 4
+        for (int r = 0; r < TB; ++r) {  // dW2: units 4 sg.., columns 4 ug..
+            const float4 d = *reinterpret_cast<const float4*>(&S.d2[r][4 * sg]);
+            const float4 h = *reinterpret_cast<const float4*>(&S.h1[r][4 * ug]);
+            const float dv[4] = {d.x, d.y, d.z, d.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) gw2[m][c] += dv[m] * hv[c];
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int r = 0; r < TB; ++r) {  // dW1: units 4 sg.., columns ug + 16 c
+            const float4 d = *reinterpret_cast<const float4*>(&S.d1[r][4 * sg]);
+            const float dv[4] = {d.x, d.y, d.z, d.w};
+            float xv[KC];
+#pragma unroll
+            for (int c = 0; c < KC; ++c) xv[c] = S.x[r][ug + 16 * c];
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int c = 0; c < KC; ++c) gw1[m][c] += dv[m] * xv[c];
+        }
+        if (t < 2 * NH) {  // db1, db2
+            const float* d = t < NH ? &S.d1[0][t] : &S.d2[0][t - NH];
+#pragma unroll 8
+            for (int r = 0; r < TB; ++r) gb += d[r * HP];
+        }
+    }
+    float* g = partial + (size_t)blockIdx.x * NPARAM;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+#pragma unroll
+        for (int c = 0; c < KC; ++c) g[O_W1 + (4 * sg + m) * NIN + ug + 16 * c] = gw1[m][c];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) g[O_W2 + (4 * sg + m) * NH + 4 * ug + c] = gw2[m][c];
+    }
+    if (t < NOUT * NH) g[O_W3 + t] = gw3;
+    else if (t < NOUT * NH + NOUT) g[O_B3 + t - NOUT * NH] = gw3;
+    if (t < NH) g[O_B1 + t] = gb;
+    else if (t < 2 * NH) g[O_B2 + t - NH] = gb;
+    // block loss (fixed-order tree)
+    for (int off = 16; off > 0; off >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, off);
+    if ((t & 31) == 0) S.red[t >> 5] = loss;
+    __syncthreads();
+    if (t == 0) {
+        float l = 0.f;
+        for (int w = 0; w < TTHR / 32; ++w) l += S.red[w];
+        lossp[blockIdx.x] = l * inv_total;
+    }
+}
+
+// Sum the per-block gradients in a fixed order (32 parameters a block, eight
+// threads a parameter taking every eighth row of the partials); then either
+// return them or take one Adam step (FP32 master, moments m, v) and refresh
+// nothing else (the BF16 copy is rebuilt by k_to_bf16).
+constexpr int kReduceParams = 32, kReduceSeg = 8;
+template <int NIN>
+__global__ void __launch_bounds__(kReduceParams * kReduceSeg)
+k_reduce_adam(const float* __restrict__ partial, const float* __restrict__ lossp, int nblk,
+              float* __restrict__ grad_out, float* __restrict__ loss_out, float* __restrict__ master,
+              float* __restrict__ m1, float* __restrict__ m2, float lr, float b1, float b2, float eps, float bc1,
+              float bc2) {
+    __shared__ float seg[kReduceSeg][kReduceParams];
     constexpr int NPARAM = Net<NIN>::NPARAM;
-    if (p >= NPARAM) return;
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int p = blockIdx.x * kReduceParams + lane;
+    float sum = 0.f;
+    if (p < NPARAM) {
+#pragma unroll 8
+        for (int b = q; b < nblk; b += kReduceSeg) sum += partial[(size_t)b * NPARAM + p];
+    }
+    seg[q][lane] = sum;
+    __syncthreads();
+    if (blockIdx.x == 0 && q == 1 && loss_out) {
+        float l = 0.f;
+        for (int b = lane; b < nblk; b += 32) l += lossp[b];
+        for (int off = 16; off > 0; off >>= 1) l += __shfl_down_sync(0xffffffffu, l, off);
+        if (lane == 0) *loss_out = l;
+    }
+    if (q != 0 || p >= NPARAM) return;
     float gsum = 0.f;
-    for (int b = 0; b < nblk; ++b) gsum += partial[(size_t)b * NPARAM + p];
+#pragma unroll
+    for (int k = 0; k < kReduceSeg; ++k) gsum += seg[k][lane];
     if (grad_out) grad_out[p] = gsum;
     if (master) {
         const float mm = b1 * m1[p] + (1.f - b1) * gsum;
@@ -1050,25 +1140,24 @@ int mlp_forward(pppm_corr* C, cudaStream_t s, const __nv_bfloat16* feat, int64_t
     return PPPM_OK;
 }
 
-template <int NIN>
-constexpr size_t grad_smem() {
-    return sizeof(float) * (NH * NIN + NH * NH + NOUT * NH + 2 * NH + 4 + TB * Net<NIN>::XP + 2 * TB * HP + TB * 4 +
-                            32);
-}
-
 int grad_step(pppm_corr* C, cudaStream_t s, const __nv_bfloat16* feat, const float* target, int64_t nrows,
               const int* idx, int64_t nb, float* grad_out, float* loss_out, bool adam, float lr) {
     if (nb <= 0 || nrows <= 0 || nb > (int64_t(1) << 30) || (!idx && nb > nrows)) return PPPM_ERR_INVALID_ARG;
-    const int nblk = (int)((nb + TB - 1) / TB);
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
+        return PPPM_ERR_CUDA;
+    // two resident blocks an SM; the tiles beyond them are looped over
+    const int nblk = (int)std::min<int64_t>((nb + TB - 1) / TB, 2 * nsm);
     int rc = ensure_partial(C, nblk);
     if (rc != PPPM_OK) return rc;
     const cudaError_t ge = with_nin(C->nin, [&](auto N) -> cudaError_t {
         constexpr int NIN = decltype(N)::value;
-        constexpr size_t smem = grad_smem<NIN>();
+        constexpr size_t smem = sizeof(GradSmem<NIN>);
         const cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<NIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)smem);
         if (e != cudaSuccess) return e;
-        k_mlp_grad<NIN><<<nblk, TB, smem, s>>>(feat, target, nrows, idx, (int)nb, 1.f / (float)nb, C->master,
+        k_mlp_grad<NIN><<<nblk, TTHR, smem, s>>>(feat, target, nrows, idx, (int)nb, 1.f / (float)nb, C->master,
                                                C->partial, C->lossp);
         return cudaGetLastError();
     });
@@ -1081,7 +1170,8 @@ int grad_step(pppm_corr* C, cudaStream_t s, const __nv_bfloat16* feat, const flo
     }
     const int npar = nparam_of(C->nin);
     with_nin(C->nin, [&](auto N) {
-        k_reduce_adam<decltype(N)::value><<<(npar + 255) / 256, 256, 0, s>>>(
+        k_reduce_adam<decltype(N)::value><<<(npar + kReduceParams - 1) / kReduceParams, kReduceParams * kReduceSeg, 0,
+                                            s>>>(
             C->partial, C->lossp, nblk, grad_out, loss_out, adam ? C->master : nullptr, C->m1, C->m2, lr, 0.9f,
             0.999f, 1e-8f, bc1, bc2);
         return 0;
