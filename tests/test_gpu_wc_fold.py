@@ -89,3 +89,28 @@ def test_fold_edge_cases(cuda_device):
     assert np.allclose(out.cpu().numpy(), ref, rtol=0, atol=1e-14)
     # zero atoms
     assert wc_fold(f[:0], 0).shape == (0, 3)
+
+
+@pytest.mark.parametrize("dt,tol", [(torch.float64, 1e-14), (torch.float32, 1e-6)])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])  # values before the Jacobian: 16-byte aligned and not
+@pytest.mark.parametrize("lengths", [(0, 1, 5, 0), (31, 32, 33, 8), (127, 0, 1, 128), (300, 2, 65, 1000), (27,) * 9])
+def test_fold_row_lengths(cuda_device, dt, tol, offset, lengths):
+    """Rows at the edges of a group's pieces and of a row's rounds, empty groups
+    between them, the last WC (whose row ends the array) included."""
+    from paper_2504_15508_gb300.pppm import wc_fold
+    rng = np.random.default_rng(sum(lengths) + offset)
+    rows = list(lengths) + [0] * 9 + list(reversed(lengths)) + [3]
+    n_atoms, n_wc = len(rows), 13
+    jp = np.concatenate([[0], np.cumsum(rows)]).astype(np.int64)
+    jw = rng.integers(0, n_wc, size=jp[-1]).astype(np.int32)
+    jw[::7] = n_wc - 1
+    J = rng.normal(size=(jp[-1], 3, 3))
+    f = rng.normal(size=(n_atoms + n_wc, 3))
+    flat = torch.empty(9 * jp[-1] + offset, dtype=dt, device="cuda")[offset:]
+    tj = flat.view(-1, 3, 3).copy_(torch.tensor(J, dtype=dt))
+    tf = torch.empty(3 * (n_atoms + n_wc) + offset, dtype=dt, device="cuda")[offset:].view(-1, 3)
+    tf.copy_(torch.tensor(f, dtype=dt))
+    out = wc_fold(tf, n_atoms, None, None, _dev(jp, torch.int64), _dev(jw, torch.int32), tj)
+    assert torch.equal(out, wc_fold(tf, n_atoms, None, None, _dev(jp, torch.int64), _dev(jw, torch.int32), tj))
+    ref = fold(tf.double().cpu().numpy(), n_atoms, None, None, jp, jw, tj.double().cpu().numpy())
+    assert np.linalg.norm(out.double().cpu().numpy() - ref) <= tol * np.linalg.norm(ref)
