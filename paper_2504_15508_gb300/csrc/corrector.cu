@@ -677,7 +677,6 @@ struct GradSmem {
     float x[TB][XP];
     float h1[TB][HP], h2[TB][HP], d1[TB][HP], d2[TB][HP];
     float dy[TB][4];
-    int site[TB];
     float red[TTHR / 32];
 };
 
@@ -714,7 +713,9 @@ __device__ __forceinline__ void tile_gemm(const float (*__restrict__ a)[AP], con
 // NIN / 16) entries of a weight gradient, so that a shared-memory wavefront
 // feeds three to five FMAs; at one thread a site (128 a block, 64 blocks at
 // 8,192 rows) each FMA read a weight of its own and less than half of the
-// SMs had a block.  8,192 rows, cell set, ncu: 77.6 -> 30.0 us.
+// SMs had a block.  8,192 rows, cell set, ncu: 77.6 -> 30.0 us.  Feature words,
+// targets and weights are asked for together before any is waited for (a tile's
+// words while the tile before it is worked on): 30.0 -> 19.3 us.
 template <int NIN>
 __global__ void __launch_bounds__(TTHR, 2)
 k_mlp_grad(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ target, int64_t nrows,
@@ -727,11 +728,49 @@ k_mlp_grad(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ tar
     GradSmem<NIN>& S = *reinterpret_cast<GradSmem<NIN>*>(sm_raw);
     const int t = threadIdx.x;
     const int ug = t & 15, sg = t >> 4;  // units 4 ug.., sites 2 sg..; in dW: columns by ug, rows 4 sg..
-    for (int i = t; i < NH * NIN; i += TTHR) S.w1t[i % NIN][i / NIN] = bfr(master[O_W1 + i]);
-    for (int i = t; i < NH * NH; i += TTHR) {
-        const float w = bfr(master[O_W2 + i]);
-        S.w2[i / NH][i % NH] = w;
-        S.w2t[i % NH][i / NH] = w;
+    // a tile's feature words (BF16 pairs) of this thread, asked for ahead of the
+    // weights: rows outside the table contribute nothing
+    constexpr int NX = TB * NIN / 2 / TTHR;
+    uint32_t xw[NX];
+    const bool words = (reinterpret_cast<uintptr_t>(feat) & 3) == 0;  // else the table starts between two words
+    auto row_of = [&](int tile, int r) {
+        const int s = tile * TB + r;
+        const int i = s < nb ? (idx ? __ldg(&idx[s]) : s) : -1;
+        return i >= 0 && i < nrows ? i : -1;
+    };
+    auto fetch = [&](int tile) {
+        int row[NX];
+#pragma unroll
+        for (int u = 0; u < NX; ++u) row[u] = row_of(tile, (t + u * TTHR) / (NIN / 2));
+#pragma unroll
+        for (int u = 0; u < NX; ++u) {
+            const __nv_bfloat16* f = feat + (int64_t)max(row[u], 0) * NIN + 2 * ((t + u * TTHR) % (NIN / 2));
+            if (row[u] < 0) xw[u] = 0u;
+            else if (words) xw[u] = __ldg(reinterpret_cast<const uint32_t*>(f));
+            else xw[u] = __ldg(reinterpret_cast<const unsigned short*>(f)) |
+                         (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(f) + 1) << 16;
+        }
+    };
+    static_assert(TB * NIN / 2 % TTHR == 0 && NH * NIN % TTHR == 0, "whole rounds of loads");
+    fetch(blockIdx.x);
+    {
+        float w1[NH * NIN / TTHR], w2[NH * NH / TTHR];
+#pragma unroll
+        for (int u = 0; u < NH * NIN / TTHR; ++u) w1[u] = master[O_W1 + t + u * TTHR];
+#pragma unroll
+        for (int u = 0; u < NH * NH / TTHR; ++u) w2[u] = master[O_W2 + t + u * TTHR];
+#pragma unroll
+        for (int u = 0; u < NH * NIN / TTHR; ++u) {
+            const int i = t + u * TTHR;
+            S.w1t[i % NIN][i / NIN] = bfr(w1[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < NH * NH / TTHR; ++u) {
+            const int i = t + u * TTHR;
+            const float w = bfr(w2[u]);
+            S.w2[i / NH][i % NH] = w;
+            S.w2t[i % NH][i / NH] = w;
+        }
     }
     for (int i = t; i < NOUT * NH; i += TTHR) S.w3[i / NH][i % NH] = bfr(master[O_W3 + i]);
     if (t < NH) {
@@ -742,20 +781,17 @@ k_mlp_grad(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ tar
     float gw1[4][KC] = {}, gw2[4][4] = {}, gw3 = 0.f, gb = 0.f, loss = 0.f;
     const int ntile = (nb + TB - 1) / TB;
     for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
-        __syncthreads();  // the previous tile has been read (the first time: the weights are in place after the next)
-        if (t < TB) {
-            const int s = tile * TB + t;
-            const int i = s < nb ? (idx ? idx[s] : s) : -1;
-            S.site[t] = i >= 0 && i < nrows ? i : -1;  // rows outside the table contribute nothing
+        __syncthreads();  // the previous tile has been read
+#pragma unroll
+        for (int u = 0; u < NX; ++u) {
+            const int i = t + u * TTHR, r = i / (NIN / 2), c = i - r * (NIN / 2);
+            *reinterpret_cast<float2*>(&S.x[r][2 * c]) =
+                make_float2(__uint_as_float(xw[u] << 16), __uint_as_float(xw[u] & 0xffff0000u));
         }
-        __syncthreads();
-        for (int i = t; i < TB * NIN / 2; i += TTHR) {  // a BF16 pair each
-            const int r = i / (NIN / 2), c = i - r * (NIN / 2), row = S.site[r];
-            float2 v = make_float2(0.f, 0.f);
-            if (row >= 0)
-                v = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(feat + (int64_t)row * NIN)[c]);
-            *reinterpret_cast<float2*>(&S.x[r][2 * c]) = v;
-        }
+        if (tile + (int)gridDim.x < ntile) fetch(tile + gridDim.x);
+        // the target of this thread's row and output (see the outputs below)
+        const int orow = row_of(tile, t >> 3);
+        const float goal = orow >= 0 && (t & 7) < NOUT ? __ldg(&target[3 * (int64_t)orow + (t & 7)]) : 0.f;
         __syncthreads();
         // hidden layers
         {
@@ -781,7 +817,7 @@ k_mlp_grad(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ tar
         }
         __syncthreads();
         {  // outputs and loss: eight threads a site, thread c < 3 of them ends with output c
-            const int r = t >> 3, c = t & 7, row = S.site[r];
+            const int r = t >> 3, c = t & 7;
             float y[NOUT] = {};
 #pragma unroll
             for (int k = c; k < NH; k += 8) {
@@ -795,7 +831,7 @@ k_mlp_grad(const __nv_bfloat16* __restrict__ feat, const float* __restrict__ tar
                 for (int o = 0; o < NOUT; ++o) y[o] += __shfl_xor_sync(0xffffffffu, y[o], h);
             if (c < NOUT) {
                 const float yc = (c == 0 ? y[0] : c == 1 ? y[1] : y[2]) + S.b3[c];
-                const float d = row >= 0 ? yc - target[3 * (int64_t)row + c] : 0.f;
+                const float d = orow >= 0 ? yc - goal : 0.f;
                 loss += d * d;
                 S.dy[r][c] = 2.f * d * inv_total;
             }
@@ -902,7 +938,7 @@ k_reduce_adam(const float* __restrict__ partial, const float* __restrict__ lossp
     const int p = blockIdx.x * kReduceParams + lane;
     float sum = 0.f;
     if (p < NPARAM) {
-#pragma unroll 8
+#pragma unroll 16
         for (int b = q; b < nblk; b += kReduceSeg) sum += partial[(size_t)b * NPARAM + p];
     }
     seg[q][lane] = sum;

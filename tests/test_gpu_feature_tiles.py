@@ -62,6 +62,10 @@ def test_gradient(cuda_device, pppm_lib, kind, nb):
     loss, g = corr.grad(feat, target, t_idx)
     loss2, g2 = corr.grad(feat, target, t_idx)
     assert torch.equal(loss, loss2) and torch.equal(g, g2)
+    # a table that starts between two 4-byte words
+    odd = torch.empty(feat.numel() + 1, dtype=torch.bfloat16, device=cuda_device)[1:].view_as(feat).copy_(feat)
+    loss3, g3 = corr.grad(odd, target, t_idx)
+    assert torch.equal(loss, loss3) and torch.equal(g, g3)
     x = feat.float().cpu().numpy().astype(np.float64)[idx]
     ref_l, ref_g = mlp.loss_and_grad(theta, x, target.cpu().numpy().astype(np.float64)[idx])
     assert abs(loss.item() - ref_l) <= 1e-5 * abs(ref_l)
