@@ -329,7 +329,9 @@ int run_sites_to_patches(pppm_plan* P, cudaStream_t s, const In* pos, const In* 
     if (region_slots(P, n) > 0) {
         // fixed tile regions: one pass over the sites; its last block rebuilds
         // the compact layout only if a region overflowed
-        { PROF(K_TILES_INIT); CK(launch_tiles_init(s, P->tiles, g.ntiles, P->region_cap, P->region_flag)); }
+        if (!one_block_sort((int)n, g.ntiles)) {
+            PROF(K_TILES_INIT); CK(launch_tiles_init(s, P->tiles, g.ntiles, P->region_cap, P->region_flag));
+        }
         DirectArgs<T> a{P->tiles, P->region_cap, P->region_flag, P->tile_of, P->slot_of,
                         (Rec<T>*)P->srec, P->scell, P->sorig, P->status};
         { PROF(K_BIN); CK((launch_bin_direct<T, In>(s, g, pos, q, (int)n, a))); }

@@ -253,7 +253,7 @@ template <int STAGE>
 static cudaError_t launch_stage(cudaStream_t s, const BoxDesc* boxes, const int2* items, int count, const Bufs& B,
                                 size_t smem) {
     auto kern = k_fft_stage<STAGE>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_k(kern, dim3(count), dim3(kThreads), smem, s, boxes, items, B);
 }

@@ -11,7 +11,7 @@ static cudaError_t run_x(cudaStream_t s, const Geo& g, const LineBlocks& lb, con
                          T e_scale, T c_field, C* S, C* Bx, T* partial) {
     auto kern = k_fft_x_reg<T, L>;
     constexpr size_t smem = x_smem<T, L>();
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_k(kern, dim3(lb.nblk), dim3(FacS<L>::NT), smem, s, g, lb, tw, G, beta, e_scale, c_field, S, Bx,
                     partial);

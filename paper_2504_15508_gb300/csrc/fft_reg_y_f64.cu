@@ -11,7 +11,7 @@ static cudaError_t run_lines(cudaStream_t s, const Geo& g, int axis, int sign, c
                              C* data) {
     auto kern = sign < 0 ? k_fft_lines<T, L, -1> : k_fft_lines<T, L, 1>;
     constexpr size_t smem = LineEngine<T, L>::kBytes;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_k(kern, dim3(lb.nblk), dim3(FacS<L>::NT), smem, s, g, axis, lb, tw, data);
 }
@@ -21,7 +21,7 @@ static cudaError_t run_inv3(cudaStream_t s, const Geo& g, const LineBlocks& lb, 
                             const T* partial, int npart, double prefactor, double* energy, double* virial) {
     auto kern = k_fft_y_inv3_reg<T, L>;
     constexpr size_t smem = 2 * LineEngine<T, L>::kBytes;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_k(kern, dim3(lb.nblk + 1), dim3(FacS<L>::NT), smem, s, g, lb, tw, A, Bx, D, partial, npart,
                     prefactor, energy, virial);

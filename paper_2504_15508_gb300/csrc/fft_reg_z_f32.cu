@@ -26,7 +26,7 @@ static cudaError_t run_r2c(cudaStream_t s, const Geo& g, const C* tw, const T* i
     const bool split = ps.patch && (int64_t)pairs * F::T < kZBlocks * 320;
     const size_t smem = sizeof(C) * F::PITCH * np;
     auto kern = split ? k_fft_z_r2c_reg<T, L, true> : k_fft_z_r2c_reg<T, L, false>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_k(kern, dim3((pairs + np - 1) / np), dim3((split ? 2 : 1) * np * F::T), smem, s, g, tw, in, out, rows, ps);
 }
@@ -39,14 +39,14 @@ static cudaError_t run_c2r(cudaStream_t s, const Geo& g, const C* tw, const ZOut
         const int np = pairs_per_block<L>(pairs, F::T, F::NPMAX);
         const size_t smem = sizeof(C) * F::PITCH * np;
         auto kern = k_fft_z_c2r_plain<T, L>;
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         return launch_k(kern, dim3((pairs + np - 1) / np, zo.nf), dim3(np * F::T), smem, s, g, tw, zo, rows);
     }
     const int np = pairs_per_block<L>(pairs, zo.nf * F::T, FacC2R<L>::NT / (zo.nf * F::T));
     const size_t smem = c2r_pair_bytes<T, L>(zo.nf) * np;
     auto kern = k_fft_z_c2r_reg<T, L>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_k(kern, dim3((pairs + np - 1) / np), dim3(np * zo.nf * F::T), smem, s, g, tw, zo, rows);
 }

@@ -260,6 +260,15 @@ __device__ __forceinline__ void split_term(float f, float twoK, int& h, int& l) 
 // 2^k from its exponent bits (-126 <= k <= 127)
 __device__ __forceinline__ float pow2f(int k) { return __uint_as_float((unsigned)(k + 127) << 23); }
 
+// Dynamic shared memory of a launch beyond what every kernel may use as it is
+// (48 KB, a little kept for the kernels' static shared memory): most launches
+// need no call here, which at nine kernels a step was 4 us of host time.
+template <typename K>
+cudaError_t allow_smem(K kern, size_t smem) {
+    if (smem <= 40 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 extern thread_local bool g_pdl;  // launches of this host thread use PDL
 
 struct PdlScope {
@@ -348,6 +357,16 @@ struct DirectArgs {
     int* status;
 };
 
+// The one-pass sort's block; up to this many sites (and kOneBlockTiles tiles, 16
+// a thread) the sort is one block that sets up the tiles itself.  A launch less:
+// 2 us of host time, and 30.7 -> 28.7 us a replayed step of 256 sites on 32^3.
+// More sites in one larger block lose that again (512: 30.8 -> 32.8 us, 1,024 on
+// 64^3: 34.3 -> 36.9).
+constexpr int kSortThreads = 256, kOneBlockTiles = 4096;
+__host__ __device__ inline bool one_block_sort(int n, int ntiles) {
+    return n > 0 && n <= kSortThreads && ntiles <= kOneBlockTiles;
+}
+
 // ------------------------------------------------------------------ launchers
 // site_sort.cu.  Tile-ordered site data are described by tiles[t] = (first
 // slot, end slot) of tile t.
@@ -360,7 +379,7 @@ cudaError_t launch_scatter(cudaStream_t s, const Geo& g, int n, const int* tile_
                            const int2* tiles, const Rec<T>* rec, const int* cell, Rec<T>* srec, int* scell,
                            int* sorig);
 // fixed regions of a.cap slots per tile: init (also zeroes the two flag words),
-// then the one-pass sort
+// then the one-pass sort; where one_block_sort holds the sort needs no init
 cudaError_t launch_tiles_init(cudaStream_t s, int2* tiles, int ntiles, int cap, int* flag);
 template <typename T, typename In>
 cudaError_t launch_bin_direct(cudaStream_t s, const Geo& g, const In* pos, const In* q, int n,

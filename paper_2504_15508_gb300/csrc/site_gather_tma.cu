@@ -274,8 +274,7 @@ static cudaError_t gather_tma(cudaStream_t s, const Geo& g, const int2* tiles, c
     const size_t smem = (4 * (size_t)E * E * EZ * sizeof(T) + 127) / 128 * 128 +
                         (kGatherWarps * 8 * WSP * sizeof(T) + 31) / 32 * 32 + kGatherWarps * 8 * 2 * sizeof(int) +
                         8;
-    cudaError_t e = cudaFuncSetAttribute(k_gather_tma<T, P, TILE, Out>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k_gather_tma<T, P, TILE, Out>, smem);
     if (e != cudaSuccess) return e;
     static const LaneRows lanes = order_rows(P, EZ);
     return launch_k(k_gather_tma<T, P, TILE, Out>, dim3(g.ntiles), dim3(kGatherWarps * 32), smem, s, g, tiles,

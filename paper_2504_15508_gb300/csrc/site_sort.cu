@@ -234,12 +234,19 @@ __global__ void k_tiles_init(int2* __restrict__ tiles, int ntiles, int cap, int*
 // The last block to finish checks the overflow flag; if a region overflowed
 // it rebuilds the compact layout alone (a scan of the counts, then every site
 // again to start + its arrival rank): slow, but only for such inputs, and no
-// extra launch on the normal path.
+// extra launch on the normal path.  A single block (one_block_sort)
+// sets up the tiles and the flag itself.
 template <typename T, typename In>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSortThreads)
 k_bin_direct(Geo g, const In* __restrict__ pos, const In* __restrict__ q, int n, DirectArgs<T> a) {
     pdl_enter();
     __shared__ bool last;
+    if (one_block_sort(n, g.ntiles)) {
+        for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) a.tiles[t] = make_int2(t * a.cap, t * a.cap);
+        if (threadIdx.x < 2) a.flag[threadIdx.x] = 0;
+        __threadfence();
+        __syncthreads();
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = i < n;
     const int lane = threadIdx.x & 31;
@@ -288,8 +295,8 @@ template <typename T, typename In>
 cudaError_t launch_bin_direct(cudaStream_t s, const Geo& g, const In* pos, const In* q, int n,
                               const DirectArgs<T>& a) {
     if (n == 0) return cudaSuccess;
-    const int blocks = (n + 255) / 256;
-    return launch_k(k_bin_direct<T, In>, dim3(blocks), dim3(256), 0, s, g, pos, q, n, a);
+    const int blocks = (n + kSortThreads - 1) / kSortThreads;
+    return launch_k(k_bin_direct<T, In>, dim3(blocks), dim3(kSortThreads), 0, s, g, pos, q, n, a);
 }
 
 // The kernels that read the sites (the nodes of a captured step whose

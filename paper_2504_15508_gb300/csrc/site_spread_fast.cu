@@ -456,7 +456,7 @@ static cudaError_t spread_fast(cudaStream_t s, const Geo& g, const int2* tiles, 
         kern = k_spread_fast<T, P, TILE>;
         smem = kSpreadWarps * sizeof(SpreadWarpSmem<T, P, TILE>);
     }
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     // as many blocks as are resident at once (the tiles beyond them go by
     // ticket): resident blocks an SM x SMs, queried once per device
