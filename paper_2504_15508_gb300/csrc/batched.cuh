@@ -15,7 +15,7 @@ constexpr int NFFT = S_ZC2R - S_ZR2C + 1;
 constexpr int kSiteChunk = 1024;  // sites per bin / scatter item
 constexpr int kZPairs = 8;        // row pairs per z-pass item, at least
 constexpr int kZRows = 512;       // and up to about this many points (pairs x Nz) an item
-constexpr int kSpreadTiles = kWarps;
+constexpr int kSpreadTiles = 2;  // tiles per spread item, one after another by the whole block
 constexpr int kGatherTiles = 2;   // four warps per tile
 
 struct BoxDesc {
