@@ -126,7 +126,9 @@ k_wc_fold_lanes(int64_t n_atoms, int64_t n_wc, const float* __restrict__ f_sites
     // a group's first block (k) and blocks (n: a row names each WC, an int, once)
     auto extent = [&](int64_t ptr, int64_t& k, int& n) {
         k = __shfl_sync(0xffffffffu, ptr, 0);
-        n = (int)min(__shfl_sync(0xffffffffu, ptr, 4) - k, (int64_t)INT_MAX);
+        const int64_t d = __shfl_sync(0xffffffffu, ptr, 4) - k;
+        n = (int)min(d, (int64_t)INT_MAX);
+        bad |= d > INT_MAX;
     };
     // the WC of block i of the n from k on (-1: none)
     auto load_wc = [&](int64_t k, int i, int n) { return i < n ? __ldg(jac_wc + k + i) : -1; };
