@@ -888,6 +888,7 @@ __device__ void st_gather(const BoxDesc& D, int idx, const Bufs& B, unsigned cha
             const bool up = (lane & h) != 0;
 #pragma unroll
             for (int i = 0; i < h; ++i) {
+                if (h >= 4 && (i & 3) == 3) continue;  // no component 3: zeros on both sides
                 const float send = up ? v[i] : v[i + h];
                 const float keep = up ? v[i + h] : v[i];
                 v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
