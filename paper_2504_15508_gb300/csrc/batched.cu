@@ -212,6 +212,23 @@ __device__ __forceinline__ void weight_row(const float4& r, float (&w)[wstride(P
     for (int a = 3 * P; a < wstride(P); ++a) w[a] = 0.f;
 }
 
+// The first P values of a weight row (16-byte aligned), read as vectors.
+template <int P>
+__device__ __forceinline__ void load_wx(const float* row, float (&wx)[8]) {
+    const float4 a = reinterpret_cast<const float4*>(row)[0];
+    wx[0] = a.x;
+    wx[1] = a.y;
+    wx[2] = a.z;
+    wx[3] = a.w;
+    if constexpr (P > 4) {
+        const float4 b = reinterpret_cast<const float4*>(row)[1];
+        wx[4] = b.x;
+        wx[5] = b.y;
+        wx[6] = b.z;
+        wx[7] = b.w;
+    }
+}
+
 template <int P, int TILE>
 __device__ void st_spread(const BoxDesc& D, int idx, const Bufs& B, unsigned char* smem) {
     typedef SpreadRed<P, TILE> L;
@@ -274,8 +291,7 @@ __device__ void st_spread(const BoxDesc& D, int idx, const Bufs& B, unsigned cha
             for (int t = warp; t < cn; t += kWarps) {
                 const float* w = rows + t * WSR;
                 float wxq[8];
-                *reinterpret_cast<float4*>(wxq) = *reinterpret_cast<const float4*>(w);
-                if constexpr (P > 4) *reinterpret_cast<float4*>(wxq + 4) = *reinterpret_cast<const float4*>(w + 4);
+                load_wx<P>(w, wxq);
                 const int cl = __float_as_int(w[WS - 1]);
                 const int lx = cl & 255, ly = (cl >> 8) & 255, lz = (cl >> 16) & 255;
                 const int base0 = lx * PLANE + ly * PZ + lz;
@@ -864,8 +880,7 @@ __device__ void st_gather(const BoxDesc& D, int idx, const Bufs& B, unsigned cha
                 const float* wj = ww + j * WSP;
                 const int base0 = lx * PLANE + ly * PZ + lz;
                 float wx[8];
-                *reinterpret_cast<float4*>(wx) = *reinterpret_cast<const float4*>(wj);
-                if constexpr (P > 4) *reinterpret_cast<float4*>(wx + 4) = *reinterpret_cast<const float4*>(wj + 4);
+                load_wx<P>(wj, wx);
 #pragma unroll
                 for (int jr = 0; jr < NR; ++jr) {
                     if (ract[jr]) {
