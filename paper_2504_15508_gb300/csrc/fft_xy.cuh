@@ -109,16 +109,18 @@ __device__ __forceinline__ void two_sum_pair(R& h, R& l, R h2, R l2) {
 
 // Sums the x pass's per-block partials (14 values a block: 7 (hi, lo) pairs)
 // in a fixed order, TwoSum in the mesh precision and hi + lo in FP64 at the
-// end, by one block of at least 32 threads.
+// end, by one block of at least 32 threads.  The sums are read past the L1: in
+// a batch other blocks of the same launch wrote them (the caller has ordered
+// their stores before this).
 template <typename R>
-__device__ __forceinline__ void finish_energy(const R* __restrict__ partial, int nblk, double prefactor,
+__device__ __forceinline__ void finish_energy(const R* partial, int nblk, double prefactor,
                                               double* __restrict__ energy, double* __restrict__ virial) {
     const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     if ((int)(threadIdx.x >> 5) >= nw) return;  // a last warp that is not whole
     for (int q = threadIdx.x >> 5; q < 7; q += nw) {
         R h = R(0), lo = R(0);
         for (int b = lane; b < nblk; b += 32)
-            two_sum_pair(h, lo, partial[(int64_t)b * 14 + 2 * q], partial[(int64_t)b * 14 + 2 * q + 1]);
+            two_sum_pair(h, lo, __ldcg(&partial[(int64_t)b * 14 + 2 * q]), __ldcg(&partial[(int64_t)b * 14 + 2 * q + 1]));
         for (int off = 16; off > 0; off >>= 1) {
             const R h2 = __shfl_down_sync(0xffffffffu, h, off);
             const R l2 = __shfl_down_sync(0xffffffffu, lo, off);

@@ -75,6 +75,28 @@ def test_staged_launch_agrees_with_persistent(cuda_device, pppm_lib):
     assert bp.launch in ("persistent", "staged") and bp.tile in (4, 8)
 
 
+def test_staged_energies_of_alternating_inputs(cuda_device, pppm_lib):
+    """The block that finishes a box's x pass sums what the box's other blocks
+    wrote in the same launch: with two inputs in turn, no sum of the call
+    before may be read, so every call's energies and virials are those of its
+    input's first call, bit for bit."""
+    from paper_2504_15508_gb300.pppm import BatchPlan
+    specs, _, pos, q, offs = _make_batch(24, seed=13, lo=64, hi=6000)
+    bp = BatchPlan(np.array([[s["L"]] * 3 for s in specs]), None, order=5, beta=0.4)
+    bp.set_launch("staged")
+    to = torch.tensor(offs, device=cuda_device)
+    tq = torch.tensor(q, device=cuda_device)
+    first = []
+    for k in range(40):
+        tp = torch.tensor(pos + np.float32(0.37 * (k % 2)), device=cuda_device)
+        e, _, v = bp.compute(tp, tq * (1 + k % 2), to)
+        if k < 2:
+            first.append((e.clone(), v.clone()))
+        else:
+            assert torch.equal(e, first[k % 2][0]) and torch.equal(v, first[k % 2][1])
+    assert bp.status() == 0 and not torch.equal(first[0][0], first[1][0])
+
+
 def test_batched_graph_replay_and_single_box_equality(cuda_device, pppm_lib):
     from paper_2504_15508_gb300.pppm import BatchPlan, Plan
     specs, boxes, pos, q, offs = _make_batch(5, seed=7)
