@@ -21,10 +21,22 @@
 // lengths up to 256 (FP64: 128) run the same passes on the register engines
 // instead (fft_reg.cuh, fft_xy.cuh, fft_z.cuh), a line's points in registers
 // with every index and radix a compile-time constant.
+#include <atomic>
+
 #include "fft_xy.cuh"
 #include "internal.cuh"
 
 namespace pppm {
+
+int device_sms() {
+    static std::atomic<int> sms[kResidentCacheDevices];  // 0: not asked yet
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 1;
+    if (dev < kResidentCacheDevices && (n = sms[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+    if (dev < kResidentCacheDevices) sms[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
 
 template <typename R>
 struct GenEngine {

@@ -186,9 +186,6 @@ struct FacZ {
     X(8) X(9) X(10) X(12) X(15) X(16) X(18) X(20) X(24) X(25) X(27) X(30) X(32) X(36) X(40) X(45) X(48) X(50) \
     X(54) X(60) X(64) X(72) X(75) X(80) X(81) X(90) X(96) X(100) X(108) X(120) X(128)
 
-// blocks the z passes aim for on small meshes, about one an SM
-constexpr int kZBlocks = 152;
-
 // resident blocks per SM of a kernel (0: it does not fit)
 template <typename K>
 int resident_blocks(K kern, int threads, size_t smem) {

@@ -10,8 +10,8 @@ typedef Cx<T>::t C;
 // block, but no less than a warp's threads
 template <int L>
 static int pairs_per_block(int pairs, int threads, int most) {
-    const int least = (32 + threads - 1) / threads;
-    int np = (pairs + kZBlocks - 1) / kZBlocks;
+    const int least = (32 + threads - 1) / threads, nsm = device_sms();
+    int np = (pairs + nsm - 1) / nsm;
     np = np < least ? least : np;
     return np > most ? most : np;
 }
@@ -23,7 +23,7 @@ static cudaError_t run_r2c(cudaStream_t s, const Geo& g, const C* tw, const T* i
     // two sets of threads fold a pair's rows while one set does not fill the
     // GPU (about 320 threads an SM): 90^3 22.0 -> 16.8 us, 64^3 12.2 -> 11.4,
     // but 128^3 16.3 -> 17.7, 160^3 25.8 -> 28.8
-    const bool split = ps.patch && (int64_t)pairs * F::T < kZBlocks * 320;
+    const bool split = ps.patch && (int64_t)pairs * F::T < device_sms() * 320;
     const size_t smem = sizeof(C) * F::PITCH * np;
     auto kern = split ? k_fft_z_r2c_reg<T, L, true> : k_fft_z_r2c_reg<T, L, false>;
     const cudaError_t e = allow_smem(kern, smem);

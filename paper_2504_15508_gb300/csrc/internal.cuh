@@ -422,6 +422,9 @@ cudaError_t launch_fft_z_r2c(cudaStream_t s, const Geo& g, const Radix& rz, cons
 template <typename T>
 cudaError_t launch_fft_bundle(cudaStream_t s, const Geo& g, int axis, int sign, const Radix& r, const LineBlocks& lb,
                               const typename Cx<T>::t* tw, typename Cx<T>::t* data);
+constexpr int kResidentCacheDevices = 64;  // devices whose figures are kept
+// SMs of the current device, asked for once per device (1 if it does not tell)
+int device_sms();
 // x FFT, influence function, inverse x FFTs; the block's energy and virial sums
 // go to partial (14 values a block), which the y inverse adds up
 template <typename T>

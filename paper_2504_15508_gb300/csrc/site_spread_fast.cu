@@ -14,7 +14,6 @@ namespace pppm {
 void upload_bspline_spread() { bsp_upload_this_unit(); }
 
 constexpr int kSpreadWarps = 4;
-constexpr int kResidentCacheDevices = 64;
 //
 // The kernels below are the ones the workloads run: tile edge and order are
 // compile-time constants (so every index is constant arithmetic) and every
