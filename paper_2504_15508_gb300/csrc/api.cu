@@ -210,7 +210,7 @@ int setup_tiles(pppm_plan* P, int T) {
         for (int d = 0; d < 3 && ok; ++d)
             for (int m = 0; m < g.N[d]; ++m) {
                 const int b = off[(size_t)d * nmax1 + m], e = off[(size_t)d * nmax1 + m + 1];
-                if (e - b > 4) { ok = false; break; }
+                if (e - b > 4 || (e - b > 2 && !near_seam(m, m, g.N[d]))) { ok = false; break; }
                 if (e - b > 2) P->cov_deep = true;
                 for (int k = b; k < e; ++k) {
                     if (d == 0) {

@@ -70,25 +70,59 @@ cudaError_t set_smem(K kernel, size_t smem) {
         _Pragma("unroll") for (int t = threadIdx.x & 31; t < (len_); t += 32)
 
 // ------------------------------------------------------------------ z forward (R2C)
-// Sum of the tile patches covering mesh point (x, y, z) (the fold of the
-// atomics-free spread) in a fixed order.
-template <typename R>
-__device__ __forceinline__ R fold_point(const Geo& g, const PatchSrc<R>& ps, int x, int y, int z) {
-    const int4 oy = __ldg(&ps.off[y]), oz = __ldg(&ps.off[ps.nmax + z]);
-    const int y4[4] = {oy.x, oy.y, oy.z, oy.w}, z4[4] = {oz.x, oz.y, oz.z, oz.w};
-    R sum = R(0);
+// Sums of the tile patches covering the points z0, z0 + 32, .. of row (x, y) (the
+// fold of the atomics-free spread) in a fixed order; 0 from point Nz on.  The
+// row's x and y entries are the same for the whole warp, and a round of loads
+// covers NP points of one (x, y) pair of covers.  Whole z forward passes with
+// this fold, with up to 64 predicated loads a point (the entries of every slot
+// read again for each), and with a fold kernel and a mesh between where a
+// length is ragged (243, 150) and eight predicated loads a point where not:
+//   FP32  288^3 244, 508, 382 us   320^3 277, 636, 481   64 x 64 x 288 27, 39, 35
+//         243^3 171, 408, 240      32 x 32 x 243 22, 54, 27
+//   FP64  144^3 162, 302, 173      192^3 356, 624, 412   64 x 64 x 150 48, 75, 46 us
+template <typename R, int NP>
+__device__ __forceinline__ void fold_points(const Geo& g, const PatchSrc<R>& ps, int row, int z0, int Nz, R (&v)[NP]) {
+    const int4* zoff = ps.off + ps.nmax + z0;
+    int2 oz[NP];
 #pragma unroll
+    for (int n = 0; n < NP; ++n) {
+        oz[n] = z0 + 32 * n < Nz ? __ldg(reinterpret_cast<const int2*>(&zoff[32 * n])) : make_int2(-1, -1);
+        v[n] = R(0);
+    }
+    const int x = row / g.N[1], y = row - x * g.N[1];
+    const int4 oy = __ldg(&ps.off[y]);
+#pragma unroll 1
     for (int a = 0; a < 4; ++a) {
         const int2 cx = __ldg(&ps.cov[4 * x + a]);
         if (cx.x < 0) break;
         const R* px = ps.patch + (int64_t)cx.x * ps.xstride + cx.y * (g.E[1] * g.Pz);
+#pragma unroll 1
+        for (int b = 0; b < 4; ++b) {
+            const int ob = b == 0 ? oy.x : b == 1 ? oy.y : b == 2 ? oy.z : oy.w;
+            if (ob < 0) break;
+            const R* py = px + ob;
+            R s0[NP], s1[NP];
 #pragma unroll
-        for (int b = 0; b < 4; ++b)
+            for (int n = 0; n < NP; ++n) s0[n] = oz[n].x >= 0 ? py[oz[n].x] : R(0);
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (y4[b] >= 0 && z4[c] >= 0) sum += px[y4[b] + z4[c]];
+            for (int n = 0; n < NP; ++n) s1[n] = oz[n].y >= 0 ? py[oz[n].y] : R(0);
+#pragma unroll
+            for (int n = 0; n < NP; ++n) {
+                v[n] += s0[n];
+                v[n] += s1[n];
+            }
+            if (ps.deep) {  // a third and fourth cover, at a ragged mesh's seam
+#pragma unroll
+                for (int n = 0; n < NP; ++n) {
+                    const int z = z0 + 32 * n;
+                    if (!near_seam(z, z, Nz) || z >= Nz) continue;
+                    const int2 d = __ldg(reinterpret_cast<const int2*>(&zoff[32 * n]) + 1);
+                    if (d.x >= 0) v[n] += py[d.x];
+                    if (d.y >= 0) v[n] += py[d.y];
+                }
+            }
+        }
     }
-    return sum;
 }
 
 template <typename R>
@@ -108,15 +142,17 @@ k_fft_z_r2c(Geo g, GenEngine<R> eng, const R* __restrict__ in, typename CT<R>::C
     const int npairs_total = (rows + 1) / 2;
     const int np = min(pairs, npairs_total - pair0);
     if (ps.patch) {
-        for (int p = threadIdx.x >> 5; p < np; p += kFftThreads >> 5) {
-            const int r0 = 2 * (pair0 + p), r1 = r0 + 1;
-            const int x0 = r0 / g.N[1], y0 = r0 - x0 * g.N[1];
-            const int x1 = r1 / g.N[1], y1 = r1 - x1 * g.N[1];
-            for (int t = threadIdx.x & 31; t < Nz; t += 32) {
-                const R va = fold_point(g, ps, x0, y0, t);
-                const R vb = r1 < rows ? fold_point(g, ps, x1, y1, t) : R(0);
-                a[t * PL + p] = CT<R>::mk(va, vb);
-            }
+        // a warp folds 32 NP points of a pair's rows at a time
+        constexpr int NP = sizeof(R) == 4 ? 4 : 2;
+        const int nch = (Nz + 32 * NP - 1) / (32 * NP);
+        for (int i = threadIdx.x >> 5; i < np * nch; i += kFftThreads >> 5) {
+            const int p = i / nch, z0 = (i - p * nch) * (32 * NP) + (threadIdx.x & 31), r0 = 2 * (pair0 + p);
+            R va[NP], vb[NP] = {};
+            fold_points<R, NP>(g, ps, r0, z0, Nz, va);
+            if (r0 + 1 < rows) fold_points<R, NP>(g, ps, r0 + 1, z0, Nz, vb);
+#pragma unroll
+            for (int n = 0; n < NP; ++n)
+                if (z0 + 32 * n < Nz) a[(z0 + 32 * n) * PL + p] = CT<R>::mk(va[n], vb[n]);
         }
     } else {
         LINE_LOOP(p, t, np, Nz) {
@@ -145,11 +181,12 @@ cudaError_t launch_fft_z_r2c(cudaStream_t s, const Geo& g, const Radix& rz, cons
     const cudaError_t re = reg_z_r2c<T>(s, g, tw, in, out, ps);
     if (re != cudaErrorNotSupported) return re;
     const int rows = g.N[0] * g.N[1];
-    // up to 15 row pairs (an odd count) per block, within 32 KB of shared memory
+    // up to 15 row pairs (an odd count) per block, within 32 KB of shared memory,
+    // and no more than give every SM a block (32 x 32 x 243: 38 -> 26 us)
     int pairs = (int)((32 * 1024) / (2 * g.N[2] * sizeof(typename Cx<T>::t)));
     pairs = pairs < 1 ? 1 : (pairs > 15 ? 15 : pairs);
-    pairs |= 1;
-    const int npairs = (rows + 1) / 2;
+    const int npairs = (rows + 1) / 2, nsm = device_sms();
+    pairs = min(pairs, (npairs + nsm - 1) / nsm) | 1;
     const size_t smem = 2ull * pairs * g.N[2] * sizeof(typename Cx<T>::t);
     auto kern = k_fft_z_r2c<T>;
     cudaError_t e = set_smem(kern, smem);

@@ -72,6 +72,14 @@ struct PatchSrc {
     int64_t xstride;   // patch elements per x tile
 };
 
+// Whether one of the indices z0 .. z1 of an axis of N points can have more than two
+// covers when order - 1 <= tile edge: only the patches of a ragged mesh's last two
+// tiles and of its first overlap so (three at most), around the seam.  setup_tiles
+// checks its lists against this.
+__host__ __device__ constexpr bool near_seam(int z0, int z1, int N) {
+    return z0 < kMaxOrder / 2 + 1 || z1 >= N - 7 - kMaxOrder / 2;
+}
+
 template <typename R> __host__ __device__ __forceinline__ R kfac(const Geo& g, int d);
 template <> __host__ __device__ __forceinline__ float kfac<float>(const Geo& g, int d) { return g.kfac_f[d]; }
 template <> __host__ __device__ __forceinline__ double kfac<double>(const Geo& g, int d) { return g.kfac_d[d]; }

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 LENGTHS = [8, 9, 10, 12, 15, 16, 18, 20, 24, 25, 27, 30, 32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 80, 81, 90, 96,
            100, 108, 120, 125, 128, 135, 144, 150, 160, 162, 180, 192, 200, 216, 225, 240, 250, 256]
-BESIDE = [5, 6, 270]  # no engine: too short, too long
+BESIDE = [5, 6, 243, 270]  # no engine: too short, no factors, too long
 DT = {"fp32": torch.float32, "fp64": torch.float64}
 TOL = {"fp32": 2e-6, "fp64": 1e-13}
 
@@ -44,7 +44,9 @@ def test_lengths(cuda_device, pppm_lib, prec, axis, length):
 @pytest.mark.parametrize("mesh,order,tile", [
     ((27, 25, 45), 5, 0), ((20, 18, 15), 4, 4), ((36, 50, 54), 7, 4),  # odd and even, two to four fold covers
     ((75, 16, 81), 6, 0), ((12, 60, 27), 3, 0), ((8, 9, 10), 5, 0),    # no room for whole tiles: the fold kernel
-    ((270, 16, 20), 5, 0), ((16, 270, 20), 5, 0), ((20, 16, 270), 5, 0)])  # one run-time axis beside two engines
+    ((270, 16, 20), 5, 0), ((16, 270, 20), 5, 0), ((20, 16, 270), 5, 0),  # one run-time axis beside two engines
+    ((16, 18, 243), 5, 8), ((18, 15, 405), 7, 8), ((12, 18, 243), 4, 4),  # run-time z, ragged: three covers
+    ((16, 25, 225), 7, 8), ((20, 16, 150), 6, 8), ((16, 16, 162), 4, 8)])  # the same where FP64 has no engine
 def test_whole_path(cuda_device, pppm_lib, prec, mesh, order, tile):
     from paper_2504_15508_gb300.pppm import Plan
     box = np.asarray(mesh) * 0.9
