@@ -95,11 +95,11 @@ __device__ __forceinline__ void run_z_r2c(const BoxDesc& D, int idx, const Bufs&
         const int n2 = j + F::T * q;
         if (!on || n2 >= F::B) continue;
         float f[F::A];
-        fold_row<float, F::A, F::B>(g, ps, 2 * pair, n2, f);
+        fold_row<float, F::A, F::B, false>(g, ps, 2 * pair, n2, f);
 #pragma unroll
         for (int n = 0; n < F::A; ++n) v[q][n] = make_float2(f[n], 0.f);
         if (two) {
-            fold_row<float, F::A, F::B>(g, ps, 2 * pair + 1, n2, f);
+            fold_row<float, F::A, F::B, false>(g, ps, 2 * pair + 1, n2, f);
 #pragma unroll
             for (int n = 0; n < F::A; ++n) v[q][n].y = f[n];
         }

@@ -15,7 +15,7 @@
 // (CUDA events around a launch, about 3 us of each figure is theirs):
 //
 //   pass                  128^3 FP32     160^3 FP32     64^3 FP64
-//   z forward with fold   24.6 -> 16.7   45.0 -> 25.6   22.5 -> 25.2 us
+//   z forward with fold   24.6 -> 16.7   45.0 -> 25.6   22.5 -> 21.4 us
 //   y forward             10.2 ->  9.8   15.2 -> 12.7   14.3 -> 11.1
 //   x and influence       25.8 -> 12.9   45.0 -> 22.3   73.6 -> 34.9
 //   y inverse, 3 outputs  16.8 -> 13.7   29.2 -> 20.1   30.6 -> 22.6
@@ -145,13 +145,15 @@ struct FacS {
 // Contiguous lines (z): two real rows a complex line; a thread of stage 2 holds
 // the frequencies k1 and A - k1 (the first one 0 and A / 2), with which every
 // mode and its Hermitian mirror lie in one thread.  A is chosen for the
-// fewest points a thread, max(A, 2 B), then for an even A.
-constexpr int paired_a(int L) {
+// fewest points a thread, max(A, 2 B), then for an even A.  A thread takes several
+// butterflies of stage 1 where that gives both stages the same threads and is no
+// more than CAP points.
+constexpr int paired_a(int L, int cap) {
     int best = 0, cost = 1 << 30;
     for (int a = 2; a <= 27; ++a) {
         if (L % a != 0 || !dft_size(a) || !dft_size(L / a)) continue;
         const int b = L / a, t2 = a / 2 + a % 2, e = a > 2 * b ? a : 2 * b;
-        const int t = b % t2 == 0 && (b / t2) * a <= 16 ? t2 : (t2 > b ? t2 : b);
+        const int t = b % t2 == 0 && (b / t2) * a <= cap ? t2 : (t2 > b ? t2 : b);
         const int c = 64 * e + 32 * (a % 2) + t;
         if (c < cost) {
             cost = c;
@@ -160,11 +162,11 @@ constexpr int paired_a(int L) {
     }
     return best;
 }
-template <int L>
+template <int L, int CAP = 16>
 struct FacZ {
-    static constexpr int A = paired_a(L), B = L / A;
+    static constexpr int A = paired_a(L, CAP), B = L / A;
     static constexpr int T2 = A / 2 + A % 2;  // threads of stage 2
-    static constexpr int T = B % T2 == 0 && (B / T2) * A <= 16 ? T2 : (T2 > B ? T2 : B);
+    static constexpr int T = B % T2 == 0 && (B / T2) * A <= CAP ? T2 : (T2 > B ? T2 : B);
     static constexpr int G1 = T < B ? B / T : 1;  // butterflies of stage 1 a thread
     static constexpr bool kWarp = 32 % T == 0;    // a line's threads share a warp
     // lines a block holds at most: about 128 threads, whole warps where T allows
@@ -174,6 +176,15 @@ struct FacZ {
     static constexpr int P0 = A * (B + 1);
     static constexpr int PITCH = P0 + ((T - P0) % 16 + 16) % 16;
 };
+
+// Points a thread of the z passes takes at most as several butterflies.  FP64: with
+// one butterfly a thread half the threads of a 100-point line have no part in stage
+// 2, and the line's ten do not share a warp: 100^3 z forward 77 -> 61 us, inverse
+// 172 -> 121.
+template <typename R>
+constexpr int kPairCap = sizeof(R) == 8 ? 20 : 16;
+template <typename R, int L>
+using FacI = FacZ<L, kPairCap<R>>;
 
 // the lengths served by the register engines
 #define PPPM_REG_LENGTHS(X)                                                                                   \

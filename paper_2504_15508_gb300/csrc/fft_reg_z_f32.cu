@@ -18,7 +18,7 @@ static int pairs_per_block(int pairs, int threads, int most) {
 
 template <int L>
 static cudaError_t run_r2c(cudaStream_t s, const Geo& g, const C* tw, const T* in, C* out, const PatchSrc<T>& ps) {
-    typedef FacZ<L> F;
+    typedef FacF<T, L> F;
     const int rows = g.N[0] * g.N[1], pairs = (rows + 1) / 2, np = pairs_per_block<L>(pairs, F::T, F::NPMAX);
     // two sets of threads fold a pair's rows while one set does not fill the
     // GPU (about 320 threads an SM): 90^3 22.0 -> 16.8 us, 64^3 12.2 -> 11.4,
@@ -33,7 +33,7 @@ static cudaError_t run_r2c(cudaStream_t s, const Geo& g, const C* tw, const T* i
 
 template <int L>
 static cudaError_t run_c2r(cudaStream_t s, const Geo& g, const C* tw, const ZOut& zo) {
-    typedef FacZ<L> F;
+    typedef FacI<T, L> F;
     const int rows = g.N[0] * g.N[1], pairs = (rows + 1) / 2;
     if (!zo.fl.padded) {
         const int np = pairs_per_block<L>(pairs, F::T, F::NPMAX);
@@ -43,7 +43,7 @@ static cudaError_t run_c2r(cudaStream_t s, const Geo& g, const C* tw, const ZOut
         if (e != cudaSuccess) return e;
         return launch_k(kern, dim3((pairs + np - 1) / np, zo.nf), dim3(np * F::T), smem, s, g, tw, zo, rows);
     }
-    const int np = pairs_per_block<L>(pairs, zo.nf * F::T, FacC2R<L>::NT / (zo.nf * F::T));
+    const int np = pairs_per_block<L>(pairs, zo.nf * F::T, FacC2R<T, L>::NT / (zo.nf * F::T));
     const size_t smem = c2r_pair_bytes<T, L>(zo.nf) * np;
     auto kern = k_fft_z_c2r_reg<T, L>;
     const cudaError_t e = allow_smem(kern, smem);

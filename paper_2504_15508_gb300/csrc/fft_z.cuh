@@ -15,10 +15,10 @@
 namespace pppm {
 
 // a line's exchange in shared memory: points (k1, n2) at k1 (B + 1) + n2
-template <typename R, int L>
-struct PairEngine : FacZ<L> {
+template <typename R, int L, int CAP = kPairCap<R>>
+struct PairEngine : FacZ<L, CAP> {
     typedef typename CT<R>::C C;
-    using F = FacZ<L>;
+    using F = FacZ<L, CAP>;
     static constexpr int A = F::A, B = F::B, T = F::T, T2 = F::T2, G1 = F::G1;
 
     // the line's other threads have written what this one reads next (every
@@ -76,8 +76,10 @@ __device__ __forceinline__ bool pair_on(int j) {
 // folded by two sets of threads: the second half of the block takes the odd
 // rows and hands them over through shared memory.
 //
-// Sum of the patches at the A points z = B n + n2 of row (x, y).
-template <typename R, int A, int B>
+// Sum of the patches at the A points z = B n + n2 of row (x, y).  SEAM: indices
+// with more than two covers lie where near_seam says, so that only those n look
+// them up (75^3 FP64 76.9 -> 62.5 us, 225^3 FP32 116 -> 91); else anywhere.
+template <typename R, int A, int B, bool SEAM>
 __device__ __forceinline__ void fold_row(const Geo& g, const PatchSrc<R>& ps, int row, int n2, R (&v)[A]) {
     const int4* zoff = ps.off + ps.nmax + n2;  // this thread's points: zoff[B n]
     int2 oz[A];
@@ -111,6 +113,7 @@ __device__ __forceinline__ void fold_row(const Geo& g, const PatchSrc<R>& ps, in
             if (ps.deep) {
 #pragma unroll
                 for (int n = 0; n < A; ++n) {
+                    if (SEAM && !near_seam(B * n, B * n + B - 1, A * B)) continue;
                     const int2 d = __ldg(reinterpret_cast<const int2*>(&zoff[B * n]) + 1);
                     if (d.x >= 0) v[n] += py[d.x];
                     if (d.y >= 0) v[n] += py[d.y];
@@ -123,11 +126,11 @@ __device__ __forceinline__ void fold_row(const Geo& g, const PatchSrc<R>& ps, in
 // The transform of a pair's rows from the points each thread holds (v[q][n] =
 // point B n + j + T q, row 0 + i row 1), and the two half rows out to o0 and
 // o0 + Hz (the second if `two`).
-template <typename R, int L>
-__device__ __forceinline__ void z_forward(typename CT<R>::C (&v)[FacZ<L>::G1][FacZ<L>::A], bool on, bool two, int j,
+template <typename R, int L, int CAP = kPairCap<R>>
+__device__ __forceinline__ void z_forward(typename CT<R>::C (&v)[FacZ<L, CAP>::G1][FacZ<L, CAP>::A], bool on, bool two, int j,
                                           typename CT<R>::C* sm, const typename CT<R>::C* __restrict__ tw,
                                           typename CT<R>::C* __restrict__ o0) {
-    typedef PairEngine<R, L> E;
+    typedef PairEngine<R, L, CAP> E;
     typedef typename CT<R>::C C;
     constexpr int A = E::A, B = E::B, T = E::T, G1 = E::G1, Hz = L / 2 + 1;
 #pragma unroll
@@ -163,14 +166,24 @@ __device__ __forceinline__ void z_forward(typename CT<R>::C (&v)[FacZ<L>::G1][Fa
     }
 }
 
+// The pass's factors: in FP64 a thread takes one butterfly of lines up to 64.  It
+// folds the points of its butterflies one after another, and a 64-point line has
+// only four threads at two each: 64^3 25.0 -> 21.3 us (22.4 for the pass staged
+// through shared memory).  The inverse keeps two, with which every thread has a
+// part of both stages (28.7 us against 41.0).
+template <typename R, int L>
+constexpr int kFoldCap = sizeof(R) == 8 && L <= 64 ? 8 : kPairCap<R>;
+template <typename R, int L>
+using FacF = FacZ<L, kFoldCap<R, L>>;
+
 template <typename R, int L, bool SPLIT>
-__global__ void __launch_bounds__((SPLIT ? 2 : 1) * FacZ<L>::T * FacZ<L>::NPMAX,
-                                  SPLIT ? pass_blocks<R, 2 * FacZ<L>::T * FacZ<L>::NPMAX>(40 + 7 * FacZ<L>::G1 * FacZ<L>::A / 2)
-                                        : pass_blocks<R, FacZ<L>::T * FacZ<L>::NPMAX>(48 + 5 * FacZ<L>::G1 * FacZ<L>::A))
+__global__ void __launch_bounds__((SPLIT ? 2 : 1) * FacF<R, L>::T * FacF<R, L>::NPMAX,
+                                  SPLIT ? pass_blocks<R, 2 * FacF<R, L>::T * FacF<R, L>::NPMAX>(40 + 7 * FacF<R, L>::G1 * FacF<R, L>::A / 2)
+                                        : pass_blocks<R, FacF<R, L>::T * FacF<R, L>::NPMAX>(48 + 5 * FacF<R, L>::G1 * FacF<R, L>::A))
 k_fft_z_r2c_reg(Geo g, const typename CT<R>::C* __restrict__ tw, const R* __restrict__ in,
                 typename CT<R>::C* __restrict__ out, int rows, PatchSrc<R> ps) {
     pdl_enter();
-    typedef PairEngine<R, L> E;
+    typedef PairEngine<R, L, kFoldCap<R, L>> E;
     typedef typename CT<R>::C C;
     constexpr int A = E::A, B = E::B, T = E::T, G1 = E::G1, Hz = L / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -192,7 +205,7 @@ k_fft_z_r2c_reg(Geo g, const typename CT<R>::C* __restrict__ tw, const R* __rest
         if (ps.patch) {
             R f[A];
             if (!odd || two) {
-                fold_row<R, A, B>(g, ps, r0 + (odd ? 1 : 0), n2, f);
+                fold_row<R, A, B, true>(g, ps, r0 + (odd ? 1 : 0), n2, f);
             } else {
 #pragma unroll
                 for (int n = 0; n < A; ++n) f[n] = R(0);
@@ -204,7 +217,7 @@ k_fft_z_r2c_reg(Geo g, const typename CT<R>::C* __restrict__ tw, const R* __rest
             }
             if constexpr (!SPLIT) {
                 if (two) {
-                    fold_row<R, A, B>(g, ps, r0 + 1, n2, f);
+                    fold_row<R, A, B, true>(g, ps, r0 + 1, n2, f);
                 } else {
 #pragma unroll
                     for (int n = 0; n < A; ++n) f[n] = R(0);
@@ -231,7 +244,7 @@ k_fft_z_r2c_reg(Geo g, const typename CT<R>::C* __restrict__ tw, const R* __rest
         }
         E::sync();  // before the line takes the hand-over's space
     }
-    z_forward<R, L>(v, on, two, j, sm, tw, out + (int64_t)r0 * Hz);
+    z_forward<R, L, kFoldCap<R, L>>(v, on, two, j, sm, tw, out + (int64_t)r0 * Hz);
 }
 
 // ------------------------------------------------------------------ z inverse (C2R)
@@ -313,7 +326,7 @@ __device__ __forceinline__ void put_point(V* out, int64_t o, int n, int n2, int 
 
 // One field (blockIdx.y) into an unpadded mesh, two rows a line.
 template <typename R, int L>
-__global__ void __launch_bounds__(FacZ<L>::T * FacZ<L>::NPMAX)
+__global__ void __launch_bounds__(FacI<R, L>::T * FacI<R, L>::NPMAX)
 k_fft_z_c2r_plain(Geo g, const typename CT<R>::C* __restrict__ tw, ZOut zo, int rows) {
     pdl_enter();
     typedef PairEngine<R, L> E;
@@ -355,16 +368,17 @@ k_fft_z_c2r_plain(Geo g, const typename CT<R>::C* __restrict__ tw, ZOut zo, int 
 // output a set 3 transforms both rows of it.
 template <typename R, int L>
 constexpr size_t c2r_pair_bytes(int nf) {
-    return sizeof(typename CT<R>::C) * FacZ<L>::PITCH * nf + 2 * L * sizeof(R) + (L % 2) * 2 * sizeof(R);
+    return sizeof(typename CT<R>::C) * FacI<R, L>::PITCH * nf + 2 * L * sizeof(R) + (L % 2) * 2 * sizeof(R);
 }
-template <int L>
+template <typename R, int L>
 struct FacC2R {  // pairs a block holds at most at three lines a pair, about 192 threads
-    static constexpr int NPMAX = FacZ<L>::T <= 32 ? 64 / FacZ<L>::T : 2, NT = 3 * FacZ<L>::T * NPMAX;
-    static constexpr int PTS = FacZ<L>::G1 * FacZ<L>::A > 2 * FacZ<L>::B ? FacZ<L>::G1 * FacZ<L>::A : 2 * FacZ<L>::B;
+    typedef FacI<R, L> F;
+    static constexpr int NPMAX = F::T <= 32 ? 64 / F::T : 2, NT = 3 * F::T * NPMAX;
+    static constexpr int PTS = F::G1 * F::A > 2 * F::B ? F::G1 * F::A : 2 * F::B;
 };
 
 template <typename R, int L>
-__global__ void __launch_bounds__(FacC2R<L>::NT, pass_blocks<R, FacC2R<L>::NT>(32 + 3 * FacC2R<L>::PTS))
+__global__ void __launch_bounds__(FacC2R<R, L>::NT, pass_blocks<R, FacC2R<R, L>::NT>(32 + 3 * FacC2R<R, L>::PTS))
 k_fft_z_c2r_reg(Geo g, const typename CT<R>::C* __restrict__ tw, ZOut zo, int rows) {
     pdl_enter();
     typedef PairEngine<R, L> E;
