@@ -470,9 +470,7 @@ void pppm_corr_destroy(pppm_corr *corr);
  *                  atom; NULL for none
  *   f_atoms        n_atoms x 3, device, written
  *   status         device int or NULL: bit 0 is set (atomically) if a WC
- *                  index was outside [0, n_wc); that entry is skipped (and,
- *                  in FP32, if the rows of four consecutive atoms hold more
- *                  than 2^31 - 1 blocks; those beyond are skipped)
+ *                  index was outside [0, n_wc); that entry is skipped
  * Row offsets must be non-decreasing and inside the arrays (not checked).
  * Asynchronous on the stream; each atom's sum has a fixed order, so the
  * result is bitwise reproducible.  The paper computes this in its MD code.

@@ -31,6 +31,7 @@
 namespace pppm {
 
 constexpr int kFoldWarps = 4;
+constexpr int kCount = 1 << 20;  // blocks of a group that are counted in 32 bits (FP32)
 constexpr int kLaneBlocks = 7, kRowBlocks = 5;  // resident blocks an SM: registers (FP32), the stages (FP64)
 
 struct FoldStage {
@@ -123,12 +124,10 @@ k_wc_fold_lanes(int64_t n_atoms, int64_t n_wc, const float* __restrict__ f_sites
         if (!jac_ptr || grp >= groups) return 0;
         return jac_ptr[min(R * grp + min(lane, R), n_atoms)];
     };
-    // a group's first block (k) and blocks (n: a row names each WC, an int, once)
+    // a group's first block (k) and blocks (n, those up to kCount)
     auto extent = [&](int64_t ptr, int64_t& k, int& n) {
         k = __shfl_sync(0xffffffffu, ptr, 0);
-        const int64_t d = __shfl_sync(0xffffffffu, ptr, 4) - k;
-        n = (int)min(d, (int64_t)INT_MAX);
-        bad |= d > INT_MAX;
+        n = (int)min(__shfl_sync(0xffffffffu, ptr, 4) - k, (int64_t)kCount);
     };
     // the WC of block i of the n from k on (-1: none)
     auto load_wc = [&](int64_t k, int i, int n) { return i < n ? __ldg(jac_wc + k + i) : -1; };
@@ -160,7 +159,7 @@ k_wc_fold_lanes(int64_t n_atoms, int64_t n_wc, const float* __restrict__ f_sites
         int b[3];
 #pragma unroll
         for (int r = 0; r < 3; ++r)
-            b[r] = (int)min(max(__shfl_sync(0xffffffffu, ptr, r + 1) - k, (int64_t)0), (int64_t)INT_MAX);
+            b[r] = (int)min(max(__shfl_sync(0xffffffffu, ptr, r + 1) - k, (int64_t)0), (int64_t)kCount);
         float acc[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) acc[i] = 0.f;
@@ -199,6 +198,27 @@ k_wc_fold_lanes(int64_t n_atoms, int64_t n_wc, const float* __restrict__ f_sites
                     acc[4 * r + 2] += c[2];
                 }
             if (last) break;
+        }
+        if (n == kCount) {  // the group's further blocks, counted in 64 bits
+            const int64_t end = __shfl_sync(0xffffffffu, ptr, 4);
+            const int64_t p1 = __shfl_sync(0xffffffffu, ptr, 1), p2 = __shfl_sync(0xffffffffu, ptr, 2),
+                          p3 = __shfl_sync(0xffffffffu, ptr, 3);
+#pragma unroll 1
+            for (int64_t q = k + n + lane; q < end; q += 32) {
+                const int m = jac_wc[q];
+                if ((unsigned)m >= nwc) {
+                    bad = true;
+                    continue;
+                }
+                const float *f = fw + 3 * (int64_t)m, *J = jac + 9 * q;
+                const int row = (q >= p1) + (q >= p2) + (q >= p3);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const float c = J[d] * f[0] + J[3 + d] * f[1] + J[6 + d] * f[2];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) acc[4 * r + d] += row == r ? c : 0.f;
+                }
+            }
         }
         // sum over the lanes: component c of row r ends in lanes 4 r + c (+ 16)
 #pragma unroll

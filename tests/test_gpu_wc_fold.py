@@ -114,3 +114,68 @@ def test_fold_row_lengths(cuda_device, dt, tol, offset, lengths):
     assert torch.equal(out, wc_fold(tf, n_atoms, None, None, _dev(jp, torch.int64), _dev(jw, torch.int32), tj))
     ref = fold(tf.double().cpu().numpy(), n_atoms, None, None, jp, jw, tj.double().cpu().numpy())
     assert np.linalg.norm(out.double().cpu().numpy() - ref) <= tol * np.linalg.norm(ref)
+
+
+def _torch_fold(f, n_atoms, hp, hw, jp, jw, J):
+    """The fold in FP64 and the sum of its terms' magnitudes, by torch's index_add."""
+    f, J, out, mag = f.double(), J.double(), f[:n_atoms].double(), f[:n_atoms].double().abs()
+    fw = f[n_atoms:]
+    rows = torch.arange(n_atoms, device="cuda")
+    ok = (jw >= 0) & (jw < fw.shape[0])
+    at = rows.repeat_interleave(jp[1:] - jp[:-1])[ok]
+    g = fw[jw[ok].long()]
+    out.index_add_(0, at, torch.einsum("kab,ka->kb", J[ok], g))
+    mag.index_add_(0, at, torch.einsum("kab,ka->kb", J[ok].abs(), g.abs()))
+    if hp is not None:
+        at = rows.repeat_interleave((hp[1:] - hp[:-1]).long())
+        out.index_add_(0, at, fw[hw.long()])
+        mag.index_add_(0, at, fw[hw.long()].abs())
+    return out, mag
+
+
+def _check_fold(dt, rows, n_wc, hosts, bad, whole=False):
+    """Rows of the given lengths; the error of a sum of m blocks of three products
+    is at most (m + 4) roundings of the terms' magnitudes, (m / 32 + 12) in FP32,
+    whose sums run over 32 lanes and then a butterfly (and a few for host terms).
+    whole: blocks and forces of small whole numbers, whose sums are exact."""
+    from paper_2504_15508_gb300.pppm import wc_fold
+    g = torch.Generator(device="cuda").manual_seed(len(rows))
+    rows = torch.as_tensor(rows, device="cuda")
+    n_atoms, zero = len(rows), torch.zeros(1, dtype=torch.int64, device="cuda")
+    jp = torch.cat([zero, rows.cumsum(0)])
+    nnz = int(jp[-1])
+    jw = torch.randint(0, n_wc, (nnz,), generator=g, device="cuda", dtype=torch.int32)
+    J = torch.randn((nnz, 3, 3), generator=g, device="cuda", dtype=dt)
+    f = torch.randn((n_atoms + n_wc, 3), generator=g, device="cuda", dtype=dt)
+    if whole:
+        J, f = J.round().clamp(-2, 2), f.round().clamp(-2, 2)
+    hp = hw = None
+    if hosts:
+        per = torch.arange(n_atoms, device="cuda") % 3  # 0, 1 or 2 hosted centroids an atom
+        hp = torch.cat([zero, per.cumsum(0)]).int()
+        hw = torch.randint(0, n_wc, (int(hp[-1]),), generator=g, device="cuda", dtype=torch.int32)
+    if bad:
+        jw[nnz // 2], jw[-1] = n_wc, -1
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = wc_fold(f, n_atoms, hp, hw, jp, jw, J, status=status)
+    assert status.item() == (1 if bad else 0)
+    assert torch.equal(out, wc_fold(f, n_atoms, hp, hw, jp, jw, J))
+    ref, mag = _torch_fold(f, n_atoms, hp, hw, jp, jw, J)
+    if whole:
+        assert torch.equal(out.double(), ref)
+        return
+    m = rows.double()[:, None]
+    bound = ((m / 32).floor() + 14) * 2.0 ** -24 if dt == torch.float32 else (m + 6) * 2.0 ** -53 * 2
+    assert bool(((out.double() - ref).abs() <= bound * mag).all())
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+def test_fold_of_more_blocks_than_counted_in_32_bits(cuda_device, dt):
+    """Rows whose group of four holds more than 2^20 blocks, which the FP32
+    kernel counts in 64 bits beyond that: one long row, alone and among short
+    ones, and a group whose second, third and fourth rows start beyond it."""
+    _check_fold(dt, [5, 2 ** 20 + 77, 0, 3], 50, True, True, whole=True)
+    rows = np.random.default_rng(4).integers(0, 9, size=60_001)
+    rows[4_000:4_004] = 3, 2 ** 20 + 77, 5, 40
+    rows[8_000:8_004] = 2 ** 20 + 1, 33, 0, 7
+    _check_fold(dt, rows, 20_000, False, True, whole=True)
