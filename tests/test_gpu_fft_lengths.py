@@ -58,7 +58,7 @@ def test_whole_path(cuda_device, pppm_lib, prec, mesh, order, tile):
     e, f, v = plan.compute(tp, tq)
     ref = OraclePPPM(box, mesh, order, 0.5).compute(tp.double().cpu().numpy(), tq.double().cpu().numpy())
     # the bars of the other parity tests
-    ftol = {"fp32": 1e-5, "fp64": 1e-12}[prec]
+    ftol, etol = {"fp32": (1e-5, 1e-6), "fp64": (1e-12, 1e-12)}[prec]
     assert np.linalg.norm(f.double().cpu().numpy() - ref["forces"]) <= ftol * np.linalg.norm(ref["forces"])
-    assert abs(e.item() - ref["energy"]) <= 1e-6 * abs(ref["energy"])
-    assert np.linalg.norm(v.cpu().numpy() - ref["virial"]) <= max(ftol, 1e-10) * np.linalg.norm(ref["virial"])
+    assert abs(e.item() - ref["energy"]) <= etol * abs(ref["energy"])
+    assert np.linalg.norm(v.cpu().numpy() - ref["virial"]) <= ftol * np.linalg.norm(ref["virial"])

@@ -60,6 +60,5 @@ def test_small_sort_replayed(cuda_device, pppm_lib, n):
         e, f, v = graph.launch(pos, q)
         graph.stream.synchronize()
         e2, f2, v2 = plan.compute(pos, q)
-        # the same terms in the arrival order of each tile's sites
-        assert torch.allclose(f, f2, rtol=0, atol=2e-5 * f2.abs().max().item())
-        assert abs(e.item() - e2.item()) <= 1e-6 * abs(e2.item()) + 1e-9
+        # each tile's sites are spread in the order of their indices, however they arrived
+        assert torch.equal(f, f2) and torch.equal(e, e2) and torch.equal(v, v2)

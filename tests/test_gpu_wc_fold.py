@@ -170,6 +170,24 @@ def _check_fold(dt, rows, n_wc, hosts, bad, whole=False):
 
 
 @pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n_atoms,mean", [
+    (17_031, 27), (17_023, 60),                                # FP32, 17,024 atoms on 152 SMs: groups of one and two
+    (34_045, 20), (34_051, 20), (34_051, 60), (34_051, 110),   # and of four; fewer where rows are long
+    (97_301, 3), (50_001, 6), (25_003, 13), (12_007, 27)])     # FP64: one, two, four and eight lanes a row
+def test_fold_groups_of_rows(cuda_device, dt, n_atoms, mean):
+    """Systems large enough that a warp takes several rows, with empty, single,
+    piece-long and long rows among them, on both sides of the lines at which
+    fewer rows share a warp; last groups that are not whole."""
+    rng = np.random.default_rng(n_atoms + mean)
+    rows = rng.integers(0, 2 * mean + 1, size=n_atoms)
+    special = rng.choice(n_atoms, size=n_atoms // 50, replace=False)
+    rows[special] = rng.choice([0, 1, 31, 32, 33, 128, 129], size=len(special))
+    rows[rng.choice(n_atoms, size=12, replace=False)] = 1000
+    rows[-3:] = 33, 0, 5
+    _check_fold(dt, rows, n_atoms // 3, True, mean % 2 == 0)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
 def test_fold_of_more_blocks_than_counted_in_32_bits(cuda_device, dt):
     """Rows whose group of four holds more than 2^20 blocks, which the FP32
     kernel counts in 64 bits beyond that: one long row, alone and among short
