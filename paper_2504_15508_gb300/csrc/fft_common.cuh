@@ -128,14 +128,15 @@ __device__ typename CT<R>::C* stockham(typename CT<R>::C* a, typename CT<R>::C* 
 
 
 
-// ------------------------------------------------------------------ compile-time engine core
-// (used by the single-box passes in fft_kernels.cu and by the batched form's
-// staged FFT kernels)
+// threads a block of the passes that stage their lines in shared memory
 constexpr int kFftThreads = 256;
 
+// ------------------------------------------------------------------ compile-time engine core
+// (used by the general FFT stages of the batched form, lines up to 64 points)
+
 // ------------------------------------------------------------------ compile-time radix plan
-// Radices 16, 10 and 8 are DFTs in registers (below), so the workload lengths
-// take two Stockham stages: 128 = 16 x 8, 160 = 16 x 10, 64 = 16 x 4, 32 = 16 x 2.
+// Radices 16, 10 and 8 are DFTs in registers (below), so that most lengths take
+// two Stockham stages: 64 = 16 x 4, 32 = 16 x 2, 40 = 10 x 4, 24 = 8 x 3.
 constexpr int fft_radix(int L, int s) {
     int m = L, i = 0;
     const int fs[7] = {16, 10, 8, 4, 2, 3, 5};

@@ -18,9 +18,9 @@
 // with sincospi and rounded to the mesh precision.
 //
 // The kernels here serve any 2^a 3^b 5^c length (radix plan read at run time);
-// lengths up to 256 (FP64: 128) run the same passes on the register engines
-// instead (fft_reg.cuh, fft_xy.cuh, fft_z.cuh), a line's points in registers
-// with every index and radix a compile-time constant.
+// those from 8 to 256 but 243 (FP64: to 128 but 125) run the same passes on the
+// register engines instead (fft_reg.cuh, fft_xy.cuh, fft_z.cuh), a line's points
+// in registers with every index and radix a compile-time constant.
 #include <atomic>
 
 #include "fft_xy.cuh"
@@ -59,10 +59,6 @@ cudaError_t set_smem(K kernel, size_t smem) {
 // lines (l) by lane within the group.
 #define BUNDLE_LOOP(t, l, L_, nl_)                                              \
     _Pragma("unroll") for (int t = threadIdx.x >> 4; t < (L_); t += kFftThreads >> 4) \
-        for (int l = threadIdx.x & 15; l < (nl_); l += 16)
-// the same without unrolling, for loop bodies too heavy to replicate
-#define BUNDLE_LOOP_ROLLED(t, l, L_, nl_)                                       \
-    _Pragma("unroll 1") for (int t = threadIdx.x >> 4; t < (L_); t += kFftThreads >> 4) \
         for (int l = threadIdx.x & 15; l < (nl_); l += 16)
 // line-major loops for the z passes: lines by warp, points by lane
 #define LINE_LOOP(line, t, nlines_, len_)                                       \

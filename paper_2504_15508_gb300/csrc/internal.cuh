@@ -58,10 +58,11 @@ struct Geo {
 // Where the forward z FFT reads its real input: a mesh, or the spread's tile
 // patches summed on the fly (the fold), through the per-axis cover lists: the
 // (tile, patch coordinate) pairs covering each mesh index, in tile order.  The
-// tables hold up to four a mesh index: two where every tile is whole, three or
-// four near the seam of a mesh whose last tile is ragged.  The x entries
-// are {tile, coordinate}, the y and z entries offsets into the patches
-// (tile part + coordinate part), -1 where there is none.
+// tables hold up to four a mesh index: two where every tile is whole, three
+// near the seam of a mesh whose last tile is ragged (in a batch also elsewhere,
+// at tile edge 4 with order 7).  The x entries are {tile, coordinate}, the y and
+// z entries offsets into the patches (tile part + coordinate part), -1 where
+// there is none.
 template <typename R>
 struct PatchSrc {
     const R* patch;    // nullptr: read the mesh

@@ -266,7 +266,7 @@ k_spread_fast(Geo g, const int2* __restrict__ tiles, const int* __restrict__ sce
 // form, plus exact zeros, so the patches are bitwise the same.
 //
 // 288,768 sites on 64^3 (4,096 tiles of 70 sites), ncu: 39.9 -> 28.7 us.  At
-// tile edge 8 the patch takes 72 registers at order 5, a third of its lanes
+// tile edge 8 the patch takes 72 registers at order 5, a quarter of its lanes
 // are padding and 16 warps an SM are left: 40.7 us against 34.6 with
 // the shared-memory patch, which therefore stays for those tiles (and for
 // FP64, whose FMAs on zero weights cost more than the wavefronts).

@@ -8,17 +8,17 @@
 // The kernels stream the blocks once (40 bytes each in FP32, 76 in FP64) and read
 // a WC force for each (12 or 24 bytes, scattered over a table that L2 holds).
 // Bound by the latency of those reads and the instructions between them: the
-// stream alone takes 34 us of the 65 for 216,576 atoms with up to 27 blocks each
+// stream alone takes 34 us of the 68 for 216,576 atoms with up to 27 blocks each
 // (72,192 molecules, FP32).  So a lane fetches the indices of its next blocks
 // while it works on the current ones, and reads a force as one or two 16-byte
 // vectors (three loads of one value each look up their cache line three times).
 //
 // The two precisions split the work differently.  In FP32 (k_wc_fold_lanes) the
 // lanes of a warp take consecutive blocks, add each to its row's accumulator,
-// and sum four rows at once with a transposing butterfly: 90.2 -> 65.9 us against
-// four xor butterflies and indices fetched when needed; rows of 0-54 blocks,
-// 100,000 atoms, 44.4 -> 39.0; of 4 blocks, 200,000 atoms, 28.8 -> 23.2 (of 200
-// blocks, 16,000 atoms, 33.3 -> 35.3: the one shape that lost).  Blocks staged through
+// and sum four rows at once with a transposing butterfly: 90.4 -> 67.8 us against
+// four xor butterflies and indices fetched when needed; 200,000 atoms of 27 blocks
+// 86.5 -> 65.8, of 4 blocks 28.9 -> 22.9, 100,000 of 0-54 43.7 -> 38.9 (16,000 of 200
+// blocks 33.9 -> 35.0: the one shape that lost).  Blocks staged through
 // shared memory took 69-92 us (fewer resident warps).  In FP64, whose additions
 // are a 64th as fast, every accumulator that a block is masked into costs
 // (27 blocks, 100,000 atoms: 327 us), so a row belongs to a set of lanes
