@@ -21,7 +21,7 @@ BOXES = {"small": [(LENGTHS[i], LENGTHS[(i + 1) % 7], LENGTHS[(i + 3) % 7]) for 
          + [(16, 25, LENGTHS[14 + i]) for i in range(7)],
          "long": [(20, 72, 16), (80, 16, 18), (18, 20, 96)],
          "six": [(6, 8, 9), (8, 6, 10), (9, 8, 6), (6, 6, 6)]}
-# order 7 on ragged and whole meshes: with tile edge 4 every index has two or three covers
+# order 7 on ragged and whole meshes: with tile edge 4 an index has two to four covers
 RAGGED = [(20, 18, 15), (12, 27, 25), (16, 20, 30), (45, 18, 50), (15, 50, 54), (24, 16, 64)]
 
 

@@ -134,9 +134,10 @@ def _torch_fold(f, n_atoms, hp, hw, jp, jw, J):
 
 
 def _check_fold(dt, rows, n_wc, hosts, bad, whole=False):
-    """Rows of the given lengths; the error of a sum of m blocks of three products
-    is at most (m + 4) roundings of the terms' magnitudes, (m / 32 + 12) in FP32,
-    whose sums run over 32 lanes and then a butterfly (and a few for host terms).
+    """Rows of the given lengths; the error of a sum of m blocks of three products,
+    up to two host terms and the atom's own is at most (m + 6) roundings of the
+    terms' magnitudes (in FP64 twice, as the reference rounds as often), and
+    (m / 32 + 14) in FP32, whose sums run over 32 lanes and then a butterfly.
     whole: blocks and forces of small whole numbers, whose sums are exact."""
     from paper_2504_15508_gb300.pppm import wc_fold
     g = torch.Generator(device="cuda").manual_seed(len(rows))
